@@ -32,7 +32,6 @@ struct SelArgs {
     int64_t nb;
     int B, k, n_sink, n_local;
     float sigma;
-    const int32_t* gate;  // nullable: the top-k runs only when *gate != 0
     int32_t* status;      // device status word (bounded waits of k_logits)
     uint64_t timeout_ns;
 };
@@ -382,7 +381,6 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
     static_assert(sizeof(whist) >= kSortMax * sizeof(uint64_t), "sort buffer");
     __shared__ uint32_t s_prefix;
     __shared__ int s_need;
-    if (a.gate && !*a.gate) return;
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
     const int u_end = unit_lower_bound(a.ut, a.sc_end);
     const int u = u_first + blockIdx.x;
@@ -680,7 +678,6 @@ __global__ void __launch_bounds__(256) k_topk_init(SelArgs a, int32_t* __restric
                                                     int32_t* __restrict__ sel_count, int32_t* __restrict__ hist,
                                                     TopkState* __restrict__ state)
 {
-    if (a.gate && !*a.gate) return;
     int u;
     int64_t lo, hi;
     if (!unit_cands(a, blockIdx.x, &u, &lo, &hi)) return;
@@ -733,7 +730,6 @@ __global__ void __launch_bounds__(kChunkThreads) k_topk_hist(SelArgs a, const fl
                                                              TopkState* __restrict__ state, int p)
 {
     __shared__ int wh[kChunkThreads / 32][256];
-    if (a.gate && !*a.gate) return;
     int u;
     int64_t lo, hi;
     if (!unit_cands(a, blockIdx.y, &u, &lo, &hi)) return;
@@ -777,7 +773,6 @@ __global__ void __launch_bounds__(kChunkThreads) k_topk_count(SelArgs a, const f
                                                               TopkState* __restrict__ state,
                                                               int2* __restrict__ counts, int max_chunks)
 {
-    if (a.gate && !*a.gate) return;
     int u;
     int64_t lo, hi;
     if (!unit_cands(a, blockIdx.y, &u, &lo, &hi)) return;
@@ -820,7 +815,6 @@ __global__ void __launch_bounds__(32) k_topk_scan(SelArgs a, const TopkState* __
                                                    int2* __restrict__ counts, int max_chunks,
                                                    int32_t* __restrict__ sel, int32_t* __restrict__ sel_count)
 {
-    if (a.gate && !*a.gate) return;
     int u;
     int64_t lo, hi;
     if (!unit_cands(a, blockIdx.x, &u, &lo, &hi)) return;
@@ -867,7 +861,6 @@ __global__ void __launch_bounds__(kChunkThreads) k_topk_emit(SelArgs a, const fl
                                                              const int2* __restrict__ counts, int max_chunks,
                                                              int32_t* __restrict__ sel)
 {
-    if (a.gate && !*a.gate) return;
     int u;
     int64_t lo, hi;
     if (!unit_cands(a, blockIdx.y, &u, &lo, &hi)) return;
@@ -1007,11 +1000,9 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
 }
 
 cudaError_t launch_topk(const Derived& d, const Units& ut, int sc_begin, int sc_end, const float* scores,
-                        int32_t* sel, int32_t* sel_count, cudaStream_t st, const int32_t* gate,
-                        const TopkScratch* scratch)
+                        int32_t* sel, int32_t* sel_count, cudaStream_t st, const TopkScratch* scratch)
 {
     SelArgs a{};
-    a.gate = gate;
     a.ut = ut;
     a.sc_begin = sc_begin;
     a.sc_end = sc_end;
