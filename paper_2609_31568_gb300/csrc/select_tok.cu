@@ -25,9 +25,11 @@
 //                   owns its (unit, token) cells, so no atomics are needed.
 //
 // Each CTA owns a tile of 128 / g units and a range of 128 g tokens (<= 1024).
-// Calls of at most 16 units (every call of the Algorithm 2 loop) use
-// k_tok_score_s instead: 16 (unit, head) columns per tile, tokens as the MMA
-// rows and the three parts side by side in one N = 48 operand.
+// Calls of at most 16 units (every call of the Algorithm 2 loop) go to score.cu:
+// one read of K, planes of logits in the workspace. Where the planes do not
+// fit there (small k with long sub-chunks) they use k_tok_score_s: 16 (unit,
+// head) columns per tile, tokens as the MMA rows and the three parts side by
+// side in one N = 48 operand.
 // Warp 0 lane 0 issues TMA loads (the fingerprint parts of one KV head, then
 // 128-token key tiles into a 2-stage ring), warp 1 lane 0 issues the MMAs
 // (TMEM: two 128-column accumulators), warps 2-5 run the epilogue. Every wait
@@ -36,6 +38,7 @@
 
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
+#include "score.cuh"
 #include "tma_host.h"
 
 namespace scale {
@@ -347,8 +350,8 @@ k_tok_score(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUte
     }
 }
 
-// ---- the same two passes for calls with few units (every call of the
-// Algorithm 2 loop covers one cluster or one sub-chunk): a unit tile of
+// ---- the same two passes for calls with few units whose planes of logits
+// (score.cu) do not fit the workspace: a unit tile of
 // 16 / G units, i.e. 16 (unit, head) columns. The 128 tokens of a key tile
 // are the MMA rows and the three bf16 parts of the 16 fingerprint columns sit
 // side by side in one N = 48 operand (part s at columns [16 s, 16 s + 16)),
@@ -822,8 +825,63 @@ cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, 
     k_tok_split<<<static_cast<unsigned>(max_units) * d.Hq, 128, 0, st>>>(a, fingerprints, parts, static_cast<int>(d.M));
     const int64_t rows = static_cast<int64_t>(max_units) * d.Hq;
     cudaError_t e = cudaSuccess;
+    // Few units (every call of the Algorithm 2 loop): one read of K with a plane
+    // of logits per unit, and the vote and the top-k in one kernel (score.cu).
+    // The planes live in the space of the packed rows, which the attention call
+    // fills later; where they do not fit (small k), K is read twice instead. Up
+    // to 16 units the planes (8 H_q bytes per token and unit, written and read)
+    // cost less than the second read of K per four units that they replace: one
+    // unit at 1M tokens 765 -> 397 us.
+    const int64_t z_stride = (d.N + 3) / 4 * 4;
+    const size_t plane = static_cast<size_t>(d.Hq) * z_stride * sizeof(float);
+    const size_t scratch_bytes = align_up(static_cast<size_t>(max_units) * kVoteScratchInts * sizeof(int32_t), kAlign);
+    if (max_units <= kSmallUnits && scratch_bytes + max_units * plane <= lay.tok_count - lay.tok_pack_k) {
+        KeyScoreArgs s{};
+        s.ut = a.ut;
+        s.sc_begin = a.sc_begin;
+        s.sc_end = a.sc_end;
+        s.Hq = d.Hq;
+        s.Hkv = d.Hkv;
+        s.N = a.N;
+        s.n_sink = d.n_sink;
+        s.n_local = d.n_local;
+        s.scale2 = a.scale2;
+        s.scratch = reinterpret_cast<int32_t*>(ws + lay.tok_pack_k);
+        s.z = reinterpret_cast<float*>(ws + lay.tok_pack_k + scratch_bytes);
+        s.z_stride = z_stride;
+        s.part = a.part;
+        s.n_part = key_logits_parts(tok_end, d.Hkv, d.M * a.n_ranges / max_units);
+        s.status = a.status;
+        s.timeout_ns = timeout_ns;
+        s.pg = pg;
+        e = launch_key_logits(s, d.g, false, parts, d.M, k, max_units, st);
+        if (e != cudaSuccess) return e;
+        VoteArgs w{};
+        w.ut = a.ut;
+        w.sc_begin = a.sc_begin;
+        w.sc_end = a.sc_end;
+        w.Hq = d.Hq;
+        w.g = d.g;
+        w.N = a.N;
+        w.k = d.k;
+        w.n_sink = d.n_sink;
+        w.n_local = d.n_local;
+        w.scale2 = a.scale2;
+        w.z = s.z;
+        w.z_stride = z_stride;
+        w.part = s.part;
+        w.n_part = s.n_part;
+        w.scores = sel_scores;
+        w.sel = sel;
+        w.sel_count = sel_count;
+        w.single = 0;
+        w.scratch = s.scratch;
+        w.gate = nullptr;
+        w.status = a.status;
+        w.timeout_ns = timeout_ns;
+        return launch_vote_topk(w, st);
+    }
     if (max_units <= kSmallUnits) {
-        // few units (every call of the Algorithm 2 loop): 16 (unit, head) columns per tile
         CUtensorMap tfs;
         const uint32_t fbox_s[4] = {64, kNc, 1, 1};
         if (!scale_host::make_dense_bf16_map(&tfs, parts, 4, fdims, fbox_s)) return cudaErrorInvalidValue;

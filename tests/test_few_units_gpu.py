@@ -1,0 +1,94 @@
+"""Token-level selection of few units (one read of K, planes of logits, vote and top-k in one launch)
+at the sizes where its tiles, slices and digits end: against the same rule in 64 bits.
+
+Scores: the dot products are exact in the three bf16 parts up to fp32 accumulation, so a logit of size
+|z| is off by a few 2^-24 |z|, which the exponential turns into the same relative error of the score:
+2e-5 holds for |z| up to about 60. A selection may differ only by tokens whose score is that close to
+the k-th one; equal keys give bit-equal scores, so exact ties have to go to the lower token.
+"""
+
+import math
+
+import pytest
+import torch
+
+import paper_2609_31568_gb300 as pkg
+from paper_2609_31568_gb300 import scale as S
+
+pytestmark = pytest.mark.gpu
+
+PER_SUB = S.SCALE_MODE_PER_SUBCHUNK
+
+# (query heads, KV heads, tokens, sub-chunk, sinks, window, k, repeated keys)
+CASES = [
+    (4, 1, 700, 100, 0, 0, 1, False),
+    (4, 1, 701, 100, 3, 50, 8, False),        # odd rows: padded planes; a sink inside the first quad
+    (4, 1, 2048, 128, 64, 128, 64, False),    # 16 units: four column tiles
+    (8, 2, 4099, 512, 130, 100, 64, True),    # exact ties across slices
+    (7, 1, 5003, 1000, 130, 64, 4999, False),  # k >= candidates
+    (5, 1, 6001, 1500, 127, 1, 300, True),
+    (3, 3, 4000, 1000, 129, 256, 2047, False),
+    (16, 16, 3000, 1000, 0, 64, 0, False),    # nothing selected
+    (1, 1, 40000, 20000, 128, 512, 19000, True),
+    (32, 8, 30011, 2048, 128, 1024, 2000, False),
+    # slices longer than the keys that stay in shared memory
+    (1, 1, 10_400_003, 5_200_064, 128, 0, 30000, False),
+]
+
+
+@pytest.fixture(scope="session", autouse=True)
+def _built():
+    pkg.build()
+    S.load()
+
+
+@pytest.mark.parametrize("hq,hkv,n,sub,sink,local,k,ties", CASES)
+def test_few_unit_token_selection(hq, hkv, n, sub, sink, local, k, ties):
+    g = hq // hkv
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    keys = torch.randn(n, hkv, 128, generator=gen, device="cuda", dtype=torch.bfloat16)
+    if ties:
+        keys = keys[:97].repeat(-(-n // 97), 1, 1)[:n].contiguous()
+    p = S.params(num_q_heads=hq, num_kv_heads=hkv, sub_chunk=sub, n_tokens=n, max_cluster_subchunks=1,
+                 block_size=1, top_k=k, n_sink=sink, n_local=local)
+    buf = pkg.allocate(p, PER_SUB, want_scores=True)
+    m = -(-n // sub)
+    fp = 0.3 * torch.randn(m, hq * 128, generator=gen, device="cuda")
+    first = max(0, m - 16)
+    for scores in (buf.sel_scores, None):  # with and without the scores asked for
+        buf.sel_blocks.fill_(-7)
+        S.scale_select_tokens(p, PER_SUB, first * sub, n, keys, fp, None, None, buf.sel_blocks, buf.sel_count,
+                              scores, buf.ws)
+        torch.cuda.synchronize()
+        assert S.scale_get_device_status(buf.ws) == S.SCALE_OK
+        for u in range(first, m):
+            w = max(0, u * sub - local)
+            cand = max(0, w - sink)
+            got = buf.sel_blocks[u, : max(k, 1)].long()
+            count = int(buf.sel_count[u])
+            assert count == min(k, cand)
+            if scores is not None:
+                off = torch.ones(n, dtype=torch.bool, device="cuda")
+                off[sink:max(w, sink)] = False
+                assert torch.equal(torch.isnan(scores[u]), off)
+            if cand == 0 or k == 0:
+                continue
+            z = torch.einsum("jgd,tjd->jgt", fp[u].view(hkv, g, 128).double(), keys[sink:w].double())
+            ref = torch.softmax(z, dim=-1).sum((0, 1))
+            if scores is not None:
+                torch.testing.assert_close(scores[u, sink:w].double(), ref, rtol=2e-5, atol=1e-10)
+            want = torch.sort(torch.sort(ref, descending=True, stable=True)[1][:k])[0] + sink
+            assert torch.all(got[count:] == -1) if count < k else True
+            assert torch.all(got[1:count] > got[: count - 1]) and got[0] >= sink and got[count - 1] < w
+            if ties:
+                # the same residues mod 97, and of the last one taken the lower tokens
+                assert torch.equal(got[:count], want) or _near(got[:count], want, ref, sink, 2e-5)
+            elif not torch.equal(got[:count], want):
+                assert _near(got[:count], want, ref, sink, 2e-5)
+
+
+def _near(got, want, ref, sink, rel):
+    """Whether every token in only one of the lists scores within `rel` of the k-th score."""
+    kth = ref[want - sink].min()
+    one = torch.cat([got[~torch.isin(got, want)], want[~torch.isin(want, got)]])
+    return bool(torch.all((ref[one - sink] / kth).log().abs() < 2 * rel)) and math.isfinite(float(kth))
