@@ -7,11 +7,11 @@
 //             into three bf16 parts, six part products accumulated in fp32)
 //   k_stats   per (u, h): max_b z and 1 / sum_b exp(z - max) over the candidates
 //   k_vote    score[u][b] = sum_h exp(z[u][h][b] - max) / sum   (heads in order)
-//   k_topk    up to 4096 candidates a bitonic sort of (score, -b) keys in
-//             shared memory, beyond that a radix select of the k-th largest
-//             key and an index-ordered compaction (and, with a scratch area
-//             and more than 64K candidates, the multi-CTA form below): output
-//             ascending, ties to the lower b.
+//   k_topk    a radix select of the k-th largest key and an index-ordered
+//             compaction (up to 4096 candidates in shared memory; with a
+//             scratch area and more than 64K candidates, the multi-CTA form
+//             below): output ascending, ties to the lower b.
+// Calls of at most 16 units run in one kernel instead, k_select_few.
 //
 // Candidates of unit u are the blocks with a token in [n_sink, W_u),
 // W_u = max(0, s_u - n_local): the contiguous range [b_lo, b_hi(u)).
@@ -306,66 +306,115 @@ __device__ __forceinline__ uint32_t float_key(float f)
 }
 
 constexpr int kTopkThreads = 1024;
-constexpr int kSortMax = 4096;     // candidates up to which the top-k sorts instead
+constexpr int kSortMax = 4096;     // candidates up to which k_topk and k_select_fused keep the keys in shared memory
 
-// The k picks among np (a power of two, at most kSortMax) 64-bit keys
-// (~float_key(score), candidate index) in shared memory, written to out in
-// ascending candidate order (candidate i is block lo + i): a bitonic sort puts
-// the picks first (higher score first, equal scores by lower index), their
-// indices are marked in a bitmap (bm: np / 32 + 1 words) and written in order
-// after one scan. Called by all kTopkThreads threads of the CTA.
-__device__ void topk_sort_emit(uint64_t* sk, uint32_t* bm, int np, int64_t lo, int k, int32_t* out)
+constexpr int kRadixBins = 2048;   // digits of 11, 11 and 10 bits
+
+// Shared memory of topk_emit.
+struct TopkShared {
+    int hist[kRadixBins];
+    int scan[32], gt[32], eq[32];
+    int digit, need;
+};
+
+// The k picks among n > k > 0 keys in shared memory (candidate i is block
+// lo + i), written to out in ascending order: a radix select of the k-th
+// largest key T (three passes over the keys, each a histogram and one block
+// scan of its bins), then the keys above T and the first ones equal to it, in
+// index order (every warp owns a run of keys: counts, one scan, ballots).
+// About 4 us for 1024 keys; the 55 exchange steps of a bitonic sort of 64-bit
+// keys took 8. Called by all THREADS threads of the CTA.
+template <int THREADS>
+__device__ void topk_emit(const uint32_t* keys, int n, int64_t lo, int k, int32_t* out, TopkShared& sh)
 {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int size = 2; size <= np; size <<= 1)
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < np; i += blockDim.x) {
-                const int l = i ^ stride;
-                if (l > i) {
-                    const uint64_t x = sk[i], y = sk[l];
-                    if ((x > y) == ((i & size) == 0)) {
-                        sk[i] = y;
-                        sk[l] = x;
-                    }
-                }
+    constexpr int kWarps = THREADS / 32;
+    constexpr int kPer = kRadixBins / THREADS;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint32_t prefix = 0;
+    int need = k;
+    for (int p = 0; p < 3; ++p) {
+        const int shift = p == 0 ? 21 : p == 1 ? 10 : 0;
+        const uint32_t mask = p == 2 ? 1023u : 2047u;
+        for (int i = tid; i < kRadixBins; i += THREADS) sh.hist[i] = 0;
+        __syncthreads();
+        for (int i = tid; i < n; i += THREADS) {
+            const uint32_t key = keys[i];
+            // the digits above this one match (p == 0: all)
+            if (p == 0 || (key >> (p == 1 ? 21 : 10)) == (prefix >> (p == 1 ? 21 : 10)))
+                atomicAdd(&sh.hist[(key >> shift) & mask], 1);
+        }
+        __syncthreads();
+        // the largest digit whose keys, with those above it, reach `need`:
+        // thread t holds kPer bins from the top, in descending order
+        const int b0 = kRadixBins - 1 - kPer * tid;
+        int h[kPer], sum = 0;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            h[e] = sh.hist[b0 - e];
+            sum += h[e];
+        }
+        int inc = sum;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane == 31) sh.scan[warp] = inc;
+        __syncthreads();
+        int before = lane < warp ? sh.scan[lane] : 0;
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+        before += inc - sum;
+#pragma unroll
+        for (int e = 0; e < kPer; ++e) {
+            if (before < need && before + h[e] >= need) {
+                sh.digit = b0 - e;
+                sh.need = need - before;
             }
-            __syncthreads();
+            before += h[e];
         }
-    for (int w = threadIdx.x; w < np / 32 + 1; w += blockDim.x) bm[w] = 0u;
-    __syncthreads();
-    for (int r = threadIdx.x; r < k; r += blockDim.x) {
-        const uint32_t i = static_cast<uint32_t>(sk[r]);
-        atomicOr(&bm[i >> 5], 1u << (i & 31));
+        __syncthreads();
+        prefix |= static_cast<uint32_t>(sh.digit) << shift;
+        need = sh.need;
+    }
+    const int run = ((n + kWarps - 1) / kWarps + 31) / 32 * 32;
+    const int r0 = warp * run, r1 = r0 + run < n ? r0 + run : n;
+    int gt = 0, eq = 0;
+    for (int i = r0 + lane; i < r1; i += 32) {
+        const uint32_t key = keys[i];
+        gt += key > prefix;
+        eq += key == prefix;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        gt += __shfl_xor_sync(0xFFFFFFFFu, gt, o);
+        eq += __shfl_xor_sync(0xFFFFFFFFu, eq, o);
+    }
+    if (lane == 0) {
+        sh.gt[warp] = gt;
+        sh.eq[warp] = eq;
     }
     __syncthreads();
-    // ascending output: word t of the bitmap to thread t, exclusive scan of the counts
-    __shared__ int s_wsum[4];
-    const int nwords = (np + 31) / 32;
-    uint32_t word = threadIdx.x < nwords ? bm[threadIdx.x] : 0u;
-    const int c = __popc(word);
-    int inc = c;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-        if (lane >= o) inc += y;
+    gt = lane < warp ? sh.gt[lane] : 0;
+    eq = lane < warp ? sh.eq[lane] : 0;
+    for (int o = 16; o > 0; o >>= 1) {
+        gt += __shfl_xor_sync(0xFFFFFFFFu, gt, o);
+        eq += __shfl_xor_sync(0xFFFFFFFFu, eq, o);
     }
-    if (lane == 31 && warp < 4) s_wsum[warp] = inc;
-    __syncthreads();
-    if (threadIdx.x < nwords) {
-        int p = inc - c;
-        for (int w = 0; w < warp; ++w) p += s_wsum[w];
-        while (word) {
-            const int bit = __ffs(word) - 1;
-            word &= word - 1;
-            out[p++] = static_cast<int32_t>(lo + 32 * threadIdx.x + bit);
-        }
+    const unsigned below = (1u << lane) - 1u;
+    for (int i0 = r0; i0 < r1; i0 += 32) {
+        const int i = i0 + lane;
+        const uint32_t key = i < r1 ? keys[i] : 0u;
+        const unsigned bg = __ballot_sync(0xFFFFFFFFu, i < r1 && key > prefix);
+        const unsigned be = __ballot_sync(0xFFFFFFFFu, i < r1 && key == prefix);
+        const int g_before = gt + __popc(bg & below), e_before = eq + __popc(be & below);
+        if ((bg >> lane & 1u) || ((be >> lane & 1u) && e_before < need))
+            out[g_before + (e_before < need ? e_before : need)] = static_cast<int32_t>(lo + i);
+        gt += __popc(bg);
+        eq += __popc(be);
     }
 }
 constexpr int kTopkUnroll = 16;  // independent loads in flight per thread
 
-// One CTA per unit. Up to kSortMax candidates, a bitonic sort in shared
-// memory of the 64-bit keys (~float_key(score), index) puts the picks first
-// (higher score first, equal scores by lower index); their indices are marked
-// in a bitmap and written in ascending order after one scan. Beyond that, the
+// One CTA per unit. Up to kSortMax candidates, topk_emit on the keys in shared
+// memory. Beyond that, the
 // k-th largest key T is found with four 8-bit radix passes (16 coalesced
 // loads in flight per thread); the selected blocks are those with key > T
 // plus the lowest-indexed ones with key == T, emitted in ascending block
@@ -377,8 +426,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
                                                        int32_t* __restrict__ sel_count)
 {
     __shared__ int hist[256];
-    __shared__ __align__(16) int whist[kTopkThreads / 32][256];  // per-warp histograms, or the sort keys
-    static_assert(sizeof(whist) >= kSortMax * sizeof(uint64_t), "sort buffer");
+    __shared__ __align__(16) int whist[kTopkThreads / 32][256];  // per-warp histograms, or keys and scratch
+    static_assert(sizeof(whist) >= kSortMax * sizeof(uint32_t) + sizeof(TopkShared), "key buffer");
     __shared__ uint32_t s_prefix;
     __shared__ int s_need;
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
@@ -399,15 +448,15 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
         return;
     }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (a.k == 0) {
+        if (threadIdx.x == 0) sel_count[u] = 0;
+        return;
+    }
     if (n <= kSortMax) {
-        uint64_t* sk = reinterpret_cast<uint64_t*>(&whist[0][0]);
-        int np = 1;
-        while (np < n) np <<= 1;
-        for (int i = threadIdx.x; i < np; i += blockDim.x)
-            sk[i] = i < n ? (static_cast<uint64_t>(~float_key(sc[lo + i])) << 32) | static_cast<uint32_t>(i)
-                          : ~0ull;  // padding sorts last
+        uint32_t* sk = reinterpret_cast<uint32_t*>(&whist[0][0]);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) sk[i] = float_key(sc[lo + i]);
         __syncthreads();
-        topk_sort_emit(sk, reinterpret_cast<uint32_t*>(hist), np, lo, a.k, out);
+        topk_emit<kTopkThreads>(sk, static_cast<int>(n), lo, a.k, out, *reinterpret_cast<TopkShared*>(sk + kSortMax));
         if (threadIdx.x == 0) sel_count[u] = a.k;  // n > k: exactly k picks
         return;
     }
@@ -551,7 +600,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
 // Steps (b)-(c) after the logits for units of at most kSortMax candidates,
 // one CTA of kTopkThreads per unit: the per-head max and 1 / sum of k_stats,
 // the soft vote of k_vote (scores written for every block, NaN off the
-// candidates) and the sort path of k_topk, with the same arithmetic in the
+// candidates) and the short path of k_topk, with the same arithmetic in the
 // same order, so scores and selection equal those of the three kernels.
 constexpr int kFusedMaxHeads = 256;
 __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const float* __restrict__ logits,
@@ -560,8 +609,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
                                                                int32_t* __restrict__ sel_count)
 {
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
-    __shared__ __align__(16) uint64_t sk[kSortMax];
-    __shared__ uint32_t bm[kSortMax / 32 + 1];
+    __shared__ uint32_t sk[kSortMax];
+    __shared__ TopkShared sh;
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
     const int u_end = unit_lower_bound(a.ut, a.sc_end);
     const int u = u_first + blockIdx.x;
@@ -602,10 +651,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
             }
         }
     __syncthreads();
-    // soft vote over the heads in order (k_vote); the candidates' sort keys
-    int np = 1;
-    while (np < n) np <<= 1;
-    const bool sort = n > a.k;
+    // soft vote over the heads in order (k_vote); the candidates' keys
+    const bool rank = n > a.k && a.k > 0;
     for (int64_t b = threadIdx.x; b < a.nb; b += kTopkThreads) {
         float score = __int_as_float(0x7FC00000);
         if (b >= lo && b < hi) {
@@ -624,21 +671,222 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
                 for (int i = 0; i < kIn; ++i)
                     if (h0 + i < a.Hq) score += expf(z[i] - mx[i]) * inv[i];
             }
-            if (sort)
-                sk[b - lo] = (static_cast<uint64_t>(~float_key(score)) << 32) | static_cast<uint32_t>(b - lo);
+            if (rank) sk[b - lo] = float_key(score);
         }
         scores[static_cast<int64_t>(u) * a.nb + b] = score;
     }
     int32_t* out = sel + static_cast<int64_t>(u) * a.k;
-    if (!sort) {
+    if (!rank) {
         for (int i = threadIdx.x; i < a.k; i += blockDim.x) out[i] = (i < n) ? static_cast<int32_t>(lo + i) : -1;
-        if (threadIdx.x == 0) sel_count[u] = static_cast<int32_t>(n);
+        if (threadIdx.x == 0) sel_count[u] = n < a.k ? static_cast<int32_t>(n) : a.k;
         return;
     }
-    for (int i = static_cast<int>(n) + threadIdx.x; i < np; i += kTopkThreads) sk[i] = ~0ull;  // padding sorts last
     __syncthreads();
-    topk_sort_emit(sk, bm, np, lo, a.k, out);
+    topk_emit<kTopkThreads>(sk, static_cast<int>(n), lo, a.k, out, sh);
     if (threadIdx.x == 0) sel_count[u] = a.k;  // n > k: exactly k picks
+}
+
+// ---- a few units (every call of the Algorithm 2 loop): the whole selection
+// in one launch.
+
+constexpr int kFewCtas = 16;       // CTAs of a unit's cluster
+constexpr int kFewThreads = 512;
+constexpr int kFewWarps = kFewThreads / 32;
+constexpr int kFewUnits = 16;      // most units per call (two rounds of the eight or nine clusters that fit at once)
+constexpr int kFewSmem = 200 * 1024;
+
+// Values v[0..V) of every lane summed over the 32 lanes: lane c ends with the
+// sum of value c % V in v[0] (halving exchanges: V - 1 shuffles, then log2(32 / V)).
+template <int V>
+__device__ __forceinline__ void reduce_to_lanes(float (&v)[V])
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int x = V / 2; x > 0; x >>= 1)
+#pragma unroll
+        for (int y = 0; y < x; ++y) {
+            const float keep = (lane & x) ? v[y + x] : v[y];
+            const float give = (lane & x) ? v[y] : v[y + x];
+            v[y] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, x);
+        }
+#pragma unroll
+    for (int x = V; x < 32; x <<= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], x);
+}
+
+// A cluster of 16 CTAs per unit, rank r owning a run of the unit's candidate
+// blocks. Logits: a warp takes NB blocks of one KV head at a time, each lane
+// four of the 128 dimensions of the representatives and of the head's G
+// queries, in fp32; they stay in shared memory. Statistics: (max, sum) of the
+// run for every head, sent to all ranks. Vote: the ranks' (max, sum) merged in
+// order, then the scores of the run, whose keys go to rank 0, which picks the
+// k largest. Nothing but the selection (and the scores, if asked for) is
+// written to memory. Bound by latency: reading 4 MB of representatives at
+// 128K tokens takes the 16 SMs about 2 us, the three exchanges and the top-k
+// the rest. A call for one unit of that layer takes 23 us from Python, most of
+// it the host's, against 35 us with k_logits and k_select_fused (16 + 15 us on
+// the GPU); 32 calls of a 32K layer take 0.43 ms less. Beyond kFewUnits the
+// 16-fold reads of the representatives and the rounds of clusters cost more
+// than the two kernels (64 units: eight rounds against 69 us).
+// Dynamic shared memory: logits [H_q][stride], then keys [nb].
+template <int G>
+__global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const float* __restrict__ fp,
+                                                               const float* __restrict__ reps, int stride,
+                                                               float* __restrict__ scores,
+                                                               int32_t* __restrict__ sel,
+                                                               int32_t* __restrict__ sel_count)
+{
+    using namespace scale_ptx;
+    constexpr int NB = G <= 4 ? 8 : 4;
+    constexpr int V = G == 1 ? 8 : G == 2 ? 16 : 32;
+    extern __shared__ float zs[];
+    __shared__ float2 s_part[kFewCtas][kFusedMaxHeads];
+    __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
+    __shared__ TopkShared sh;
+    const int u = unit_lower_bound(a.ut, a.sc_begin) + static_cast<int>(blockIdx.y);
+    if (u >= unit_lower_bound(a.ut, a.sc_end)) return;  // the whole cluster
+    int anc;
+    int64_t s, e, lo, hi;
+    unit_range(a.ut, u, &anc, &s, &e);
+    cand_range(a, s, &lo, &hi);
+    const int n = static_cast<int>(hi - lo);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = static_cast<int>(cluster_ctarank());
+    float* sc = scores ? scores + static_cast<int64_t>(u) * a.nb : nullptr;
+    int32_t* out = sel + static_cast<int64_t>(u) * a.k;
+    if (sc)  // NaN off the candidates
+        for (int64_t b = rank * kFewThreads + tid; b < a.nb; b += kFewCtas * kFewThreads)
+            if (b < lo || b >= hi) sc[b] = __int_as_float(0x7FC00000);
+    const bool pick = n > a.k && a.k > 0;
+    if (!pick) {  // every candidate, or none
+        if (rank == 0) {
+            for (int i = tid; i < a.k; i += kFewThreads) out[i] = i < n ? static_cast<int32_t>(lo + i) : -1;
+            if (tid == 0) sel_count[u] = n < a.k ? n : a.k;
+        }
+        if (!sc || n == 0) return;
+    }
+    cluster_arrive();  // waited for before the first store to another rank: all have started
+    const int slice = ((n + kFewCtas - 1) / kFewCtas + NB - 1) / NB * NB;  // at most `stride`
+    const int r0 = rank * slice;
+    const int len = n - r0 < slice ? (n - r0 > 0 ? n - r0 : 0) : slice;
+    const int Hkv = a.Hq / G;
+
+    // logits of the run: items (KV head, NB blocks), a KV head's items on neighbouring warps
+    const int nbk = (len + NB - 1) / NB;
+    for (int it = warp; it < nbk * Hkv; it += kFewWarps) {
+        const int j = it / nbk, b0 = (it - j * nbk) * NB;
+        const float4* rp = reinterpret_cast<const float4*>(reps + (j * a.nb + lo + r0 + b0) * kHeadDim) + lane;
+        float4 x[NB];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            x[i] = b0 + i < len ? __ldg(rp + i * (kHeadDim / 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4* qp = reinterpret_cast<const float4*>(fp + (static_cast<int64_t>(anc) * a.Hq + j * G) * kHeadDim) + lane;
+        float v[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) v[i] = 0.f;
+#pragma unroll
+        for (int hl = 0; hl < G; ++hl) {
+            const float4 qv = __ldg(qp + hl * (kHeadDim / 4));
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                v[hl * NB + i] = fmaf(qv.x, x[i].x, qv.y * x[i].y) + fmaf(qv.z, x[i].z, qv.w * x[i].w);
+        }
+        reduce_to_lanes<V>(v);
+        if (lane < G * NB) zs[(j * G + lane / NB) * stride + b0 + lane % NB] = a.sigma * v[0];
+    }
+    cluster_wait();
+    __syncthreads();
+    // (max, sum) of the run per head, to every rank: lane x sends to rank x % 16
+    for (int h = warp; h < a.Hq; h += kFewWarps) {
+        float m = -INFINITY, sum = 0.f;
+        for (int i = lane; i < len; i += 32) m = fmaxf(m, zs[h * stride + i]);
+        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+        for (int i = lane; i < len; i += 32) sum += expf(zs[h * stride + i] - m);
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        if (lane < kFewCtas) st_cluster_f2(cluster_map(&s_part[rank][h], lane), m, sum);
+    }
+    cluster_arrive();
+    cluster_wait();
+    for (int h = tid; h < a.Hq; h += kFewThreads) {
+        float m = -INFINITY, sum = 0.f;
+#pragma unroll
+        for (int r = 0; r < kFewCtas; ++r) m = fmaxf(m, s_part[r][h].x);
+#pragma unroll
+        for (int r = 0; r < kFewCtas; ++r)
+            if (s_part[r][h].x > -INFINITY) sum += s_part[r][h].y * expf(s_part[r][h].x - m);
+        s_m[h] = m;
+        s_inv[h] = 1.0f / sum;
+    }
+    __syncthreads();
+    uint32_t* keys = reinterpret_cast<uint32_t*>(zs + static_cast<size_t>(a.Hq) * stride);
+    const uint32_t keys0 = cluster_map(keys, 0);
+    for (int i = tid; i < len; i += kFewThreads) {
+        float score = 0.f;
+        for (int h = 0; h < a.Hq; ++h) score += expf(zs[h * stride + i] - s_m[h]) * s_inv[h];
+        if (sc) sc[lo + r0 + i] = score;
+        if (pick) st_cluster_u32(keys0 + 4 * (r0 + i), float_key(score));
+    }
+    cluster_arrive();  // after it rank 0 has every key and no rank's shared memory is written
+    cluster_wait();
+    if (rank != 0 || !pick) return;
+    topk_emit<kFewThreads>(keys, n, lo, a.k, out, sh);
+    if (tid == 0) sel_count[u] = a.k;
+}
+
+// Shared memory of k_select_few for these parameters, 0 when it does not fit
+// (or the shapes are outside it): the three kernels serve those.
+struct FewPlan {
+    int stride;
+    size_t smem;
+};
+FewPlan few_plan(const Derived& d, int max_units)
+{
+    FewPlan p{0, 0};
+    if (max_units > kFewUnits || d.g > 8 || d.Hq > kFusedMaxHeads) return p;
+    const int64_t stride = ((d.nb + kFewCtas - 1) / kFewCtas + 7) / 8 * 8;
+    const int64_t bytes = (stride * d.Hq + d.nb) * 4;
+    if (bytes > kFewSmem - 48 * 1024) return p;
+    p.stride = static_cast<int>(stride);
+    p.smem = static_cast<size_t>(bytes);
+    return p;
+}
+
+template <int G>
+cudaError_t run_select_few(const SelArgs& a, const FewPlan& p, int max_units, const float* fp, const float* reps,
+                           float* scores, int32_t* sel, int32_t* sel_count, cudaStream_t st)
+{
+    // set on every launch: the attributes belong to the current device
+    cudaError_t e = cudaFuncSetAttribute(k_select_few<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(p.smem));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_few<G>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(kFewCtas, static_cast<unsigned>(max_units));
+    cfg.blockDim = dim3(kFewThreads);
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kFewCtas;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_select_few<G>, a, fp, reps, p.stride, scores, sel, sel_count);
+}
+
+cudaError_t launch_select_few(const Derived& d, const SelArgs& a, const FewPlan& p, int max_units, const float* fp,
+                              const float* reps, float* scores, int32_t* sel, int32_t* sel_count, cudaStream_t st)
+{
+    switch (d.g) {
+    case 1: return run_select_few<1>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 2: return run_select_few<2>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 3: return run_select_few<3>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 4: return run_select_few<4>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 5: return run_select_few<5>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 6: return run_select_few<6>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 7: return run_select_few<7>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    default: return run_select_few<8>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    }
 }
 
 // ---- top-k over many candidates per unit: the same radix select and ordered
@@ -980,6 +1228,15 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
     const int max_units = a.sc_end - a.sc_begin;  // units in range <= sub-chunks in range
     if (max_units <= 0) return cudaSuccess;
 
+    const FewPlan few = few_plan(d, max_units);
+    if (few.stride) {
+        // A cluster of 16 may not be had everywhere (a partition of the device);
+        // nothing is enqueued then and the kernels below do the work.
+        const cudaError_t ef = launch_select_few(d, a, few, max_units, fingerprints, reps, sel_scores, sel_blocks,
+                                                 sel_count, st);
+        if (ef == cudaSuccess) return ef;
+        cudaGetLastError();
+    }
     const int upt = 128 / d.g;  // units per logits tile
     // set on every launch: the attribute belongs to the current device
     cudaError_t e = cudaFuncSetAttribute(k_logits, cudaFuncAttributeMaxDynamicSharedMemorySize,

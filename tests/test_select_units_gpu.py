@@ -1,0 +1,93 @@
+"""Block-level selection against the same rule in 64 bits, at the sizes where the few-unit kernel's
+runs, groups and cluster end and on both sides of the line to the kernels for many units.
+
+Scores: the error of a logit is the relative error of the score. The tensor-core kernel adds 48 partial
+products per logit into an fp32 accumulator, each addition off by at most 2^-23 (truncation) of a partial
+sum, taken as at most the largest logit: 48 * 2^-23 * max|z|. The few-unit kernel's fp32 sums of 128
+products in trees stay far below that. A selection may differ only by blocks whose score is that close to
+the k-th one; equal representatives give bit-equal scores, so exact ties have to go to the lower block.
+"""
+
+import pytest
+import torch
+
+import paper_2609_31568_gb300 as pkg
+from paper_2609_31568_gb300 import scale as S
+
+pytestmark = pytest.mark.gpu
+
+PER_SUB = S.SCALE_MODE_PER_SUBCHUNK
+
+# (query heads, KV heads, tokens, sub-chunk, block, sinks, window, k, units of the call, repeated rows)
+CASES = [
+    (4, 1, 1100, 64, 8, 0, 0, 1, 16, False),
+    (4, 1, 1100, 64, 8, 0, 0, 1, 18, False),        # one more unit than a call of the few-unit kernel
+    (1, 1, 4000, 1000, 3, 5, 17, 100, 4, True),     # ragged blocks, exact ties across the ranks
+    (2, 1, 4000, 1000, 16, 16, 100, 249, 4, False),  # k = candidates - 1 and candidates for some units
+    (3, 1, 5000, 500, 7, 40, 100, 33, 9, False),
+    (5, 1, 5000, 500, 7, 40, 100, 33, 10, True),
+    (12, 2, 5000, 1000, 9, 0, 1, 64, 5, False),
+    (28, 4, 8200, 1024, 33, 64, 128, 20, 9, False),
+    (64, 8, 8200, 1024, 64, 64, 128, 20, 8, True),
+    (256, 64, 3000, 1000, 64, 64, 128, 8, 3, False),  # the most heads of the fused kernels
+    (260, 52, 3000, 1000, 64, 64, 128, 8, 3, False),  # and beyond
+    (10, 1, 3000, 1000, 32, 0, 0, 8, 3, False),       # group of 10: the kernels for many units
+    (4, 1, 40000, 10000, 10, 0, 0, 4000, 4, False),   # 4000 blocks
+    (32, 8, 70000, 10000, 16, 64, 128, 1000, 7, True),  # more blocks than the shared memory holds
+    (4, 2, 3000, 1000, 64, 64, 128, 0, 3, False),     # nothing selected
+    (4, 1, 300000, 10000, 64, 64, 1024, 64, 30, True),  # many units, 4,688 blocks
+]
+
+
+@pytest.fixture(scope="session", autouse=True)
+def _built():
+    pkg.build()
+    S.load()
+
+
+@pytest.mark.parametrize("hq,hkv,n,sub,block,sink,local,k,units,ties", CASES)
+def test_block_selection_of_units(hq, hkv, n, sub, block, sink, local, k, units, ties):
+    g, m, nb = hq // hkv, -(-n // sub), -(-n // block)
+    gen = torch.Generator(device="cuda").manual_seed(n + hq)
+    reps = torch.randn(hkv, nb, 128, generator=gen, device="cuda")
+    if ties:
+        reps = reps[:, :61].repeat(1, -(-nb // 61), 1)[:, :nb].contiguous()
+    fp = 0.3 * torch.randn(m, hq * 128, generator=gen, device="cuda")
+    p = S.params(num_q_heads=hq, num_kv_heads=hkv, sub_chunk=sub, n_tokens=n, max_cluster_subchunks=1,
+                 block_size=block, top_k=k, n_sink=sink, n_local=local)
+    buf = pkg.allocate(p, PER_SUB, want_scores=True)
+    first = max(0, m - units)
+    for scores in (buf.sel_scores, None):  # with and without the scores asked for
+        buf.sel_blocks.fill_(-7)
+        S.scale_select(p, PER_SUB, first * sub, n, reps, fp, None, None, buf.sel_blocks, buf.sel_count, scores, buf.ws)
+        torch.cuda.synchronize()
+        assert S.scale_get_device_status(buf.ws) == S.SCALE_OK
+        for u in range(first, m):
+            lo = sink // block
+            hi = max(lo, -(-max(0, u * sub - local) // block))
+            count = int(buf.sel_count[u])
+            assert count == min(k, hi - lo)
+            if scores is not None:
+                off = torch.ones(nb, dtype=torch.bool, device="cuda")
+                off[lo:hi] = False
+                assert torch.equal(torch.isnan(scores[u]), off)
+            if hi == lo or k == 0:
+                continue
+            z = torch.einsum("jgd,jbd->jgb", fp[u].view(hkv, g, 128).double(), reps[:, lo:hi].double())
+            ref = torch.softmax(z, dim=-1).sum((0, 1))
+            tol = 48 * 2.0 ** -23 * max(1.0, float(z.abs().max()))
+            if scores is not None:
+                torch.testing.assert_close(scores[u, lo:hi].double(), ref, rtol=tol, atol=1e-10)
+            got = buf.sel_blocks[u, :k].long()
+            want = torch.sort(torch.sort(ref, descending=True, stable=True)[1][:k])[0] + lo
+            assert torch.all(got[count:] == -1)
+            got = got[:count]
+            assert torch.all(got[1:] > got[:-1]) and got[0] >= lo and got[-1] < hi
+            if not torch.equal(got, want):
+                kth = ref[want - lo].min()
+                one = torch.cat([got[~torch.isin(got, want)], want[~torch.isin(want, got)]])
+                assert torch.all((ref[one - lo] / kth).log().abs() < 2 * tol)
+                if ties:  # of a tied group that is cut, the lower blocks
+                    for r in torch.unique((one - lo) % 61):
+                        mine = got[(got - lo) % 61 == r]
+                        assert torch.equal(mine, torch.arange(len(mine), device="cuda") * 61 + r + lo)
