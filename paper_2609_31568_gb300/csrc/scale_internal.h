@@ -16,6 +16,7 @@ constexpr int kHeadDim = 128;
 constexpr int kSegRows = 64;         // rows of one K/V TMA box (a "segment")
 constexpr int kMaxSegments = 1024;   // distant segments per unit the attention kernel can hold
 constexpr int kStatusOffset = 0;     // device status word (int32) at the start of the workspace
+constexpr int kTicketOffset = 64;    // CTA ticket of step (a), in the same 256 bytes
 constexpr size_t kAlign = 256;
 
 // Device status word values: 0, SCALE_ERR_TIMEOUT, SCALE_ERR_DEVICE.
