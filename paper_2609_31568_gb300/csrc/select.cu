@@ -3,7 +3,7 @@
 // instantiation") over block representative keys, then a deterministic top-k.
 //
 //   k_logits  z[u][h][b] = sigma * v_a(u)^(h) . r_b^(h/g)   (tcgen05 MMA per KV head:
-//             128 (unit, head) rows x 128 blocks; both fp32 operands split
+//             128 blocks x 64 (unit, head) rows; both fp32 operands split
 //             into three bf16 parts, six part products accumulated in fp32)
 //   k_stats   per (u, h): max_b z and 1 / sum_b exp(z - max) over the candidates
 //   k_vote    score[u][b] = sum_h exp(z[u][h][b] - max) / sum   (heads in order)
@@ -45,22 +45,30 @@ __device__ __forceinline__ void cand_range(const SelArgs& a, int64_t s, int64_t*
     if (*hi < *lo) *hi = *lo;
 }
 
-// Tensor-core logits. Grid: (unit tiles of 128 / g units, 128-block tiles,
-// KV heads j). Rows of the A operand are the (unit, query head of KV head j)
-// pairs of the tile (row ul * g + hl: head j g + hl of unit u0 + ul, the
-// anchor's fingerprint slice), columns of B are the representatives of blocks
-// [b0, b0 + 128) of KV head j. Both are fp32; every value x is split into
-// three bf16 parts x1 + x2 + x3 = x exactly (x1 = bf16(x), x2 = bf16(x - x1),
-// x3 = x - x1 - x2), written by the threads straight into the 128-byte-
-// swizzled K-major layout of the MMA. The six part products a_i b_j with
-// i + j <= 4 are exact in fp32 and are accumulated in fp32 in TMEM; the three
-// dropped ones are below 2^-24 of |a| |b|. Only candidate blocks of each row's
-// unit are written, as before.
-constexpr int kLtThreads = 256;
-constexpr uint32_t kLtPart = 128 * 128 * 2;   // one bf16 part: 128 rows x 128 columns
-constexpr uint32_t kLtHalf = kLtPart / 2;     // one 64-column half
-constexpr uint32_t kLtSmem = 6 * kLtPart + 1024;
-static_assert(kLtSmem <= 227 * 1024, "logits shared memory");
+// Tensor-core logits. A CTA owns 128 blocks of one KV head j and walks a
+// segment of the call's unit tiles (64 (unit, query head of j) rows: row
+// ul * g + hl is head j g + hl of unit ul of the tile, the anchor's fingerprint
+// slice). The representatives are the MMA's rows (TMEM lanes), so a warp stores
+// 32 consecutive blocks of a logit row at a time; they are staged once per CTA,
+// the fingerprint rows once per tile into one of two buffers. Both are fp32;
+// every value x is split into three bf16 parts x1 + x2 + x3 = x exactly (x1 =
+// bf16(x), x2 = bf16(x - x1), x3 = x - x1 - x2), written by the threads straight
+// into the 128-byte-swizzled K-major layout of the MMA. The six part products
+// a_i b_j with i + j <= 4 are exact in fp32 and are accumulated in fp32 in TMEM;
+// the three dropped ones are below 2^-24 of |a| |b|. Only candidate blocks of
+// each row's unit are written. Warp 0 lane 0 issues the MMAs (two accumulators
+// of 64 columns), warps 1-4 store, warps 5-12 load and split the next tile: the
+// three overlap, and what bounds the kernel is the staging of a tile. 256
+// units x 4,096 blocks x 32 heads: 81 us (one CTA per tile, staging both
+// operands each time and nothing overlapped: 185 us).
+constexpr int kLtStageThreads = 256;
+constexpr int kLtThreads = 32 + 128 + kLtStageThreads;
+constexpr int kLtRows = 64;                        // (unit, head) rows of a tile
+constexpr int kLtSeg = 8;                          // most tiles of a CTA
+constexpr uint32_t kLtBPart = 128 * 128 * 2;       // one bf16 part of the representatives
+constexpr uint32_t kLtAPart = kLtRows * 128 * 2;   // one bf16 part of a tile's rows
+constexpr uint32_t kLtSmem = 3 * kLtBPart + 2 * 3 * kLtAPart + 1024;
+static_assert(kLtSmem + kLtSeg * kLtRows * 8 + 1024 <= 227 * 1024, "logits shared memory");
 
 __device__ __forceinline__ void split_bf16x3(float x, __nv_bfloat16& p1, __nv_bfloat16& p2, __nv_bfloat16& p3)
 {
@@ -71,8 +79,9 @@ __device__ __forceinline__ void split_bf16x3(float x, __nv_bfloat16& p1, __nv_bf
 }
 
 // Four consecutive fp32 values of row r, columns [c, c + 4), into the three
-// bf16 parts at `base` (part s at base + s * kLtPart): 8 bytes per part, at
-// the 128-byte-swizzled K-major position of (r, c).
+// bf16 parts at `base` (part s at base + s * PART, of two 64-column halves): 8
+// bytes per part, at the 128-byte-swizzled K-major position of (r, c).
+template <uint32_t PART>
 __device__ __forceinline__ void put_split4(uint8_t* base, int r, int c, float4 v)
 {
     __nv_bfloat16 p[3][4];
@@ -81,7 +90,7 @@ __device__ __forceinline__ void put_split4(uint8_t* base, int r, int c, float4 v
     split_bf16x3(v.z, p[0][2], p[1][2], p[2][2]);
     split_bf16x3(v.w, p[0][3], p[1][3], p[2][3]);
     const int hf = c >> 6, cc = c & 63;  // half, column in the half
-    const uint32_t off = hf * kLtHalf + (r >> 3) * 1024 + (r & 7) * 128 + ((((cc >> 3) ^ (r & 7))) << 4) +
+    const uint32_t off = hf * (PART / 2) + (r >> 3) * 1024 + (r & 7) * 128 + ((((cc >> 3) ^ (r & 7))) << 4) +
                          (cc & 7) * 2;
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
@@ -90,71 +99,87 @@ __device__ __forceinline__ void put_split4(uint8_t* base, int r, int c, float4 v
               (static_cast<uint32_t>(__bfloat16_as_ushort(p[s][1])) << 16);
         w.y = static_cast<uint32_t>(__bfloat16_as_ushort(p[s][2])) |
               (static_cast<uint32_t>(__bfloat16_as_ushort(p[s][3])) << 16);
-        *reinterpret_cast<uint2*>(base + s * kLtPart + off) = w;
+        *reinterpret_cast<uint2*>(base + s * PART + off) = w;
     }
 }
 
-__global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, const float* __restrict__ fp,
+struct LtBars {
+    uint64_t a_full[2], a_empty[2];
+    uint64_t d_full[2], d_empty[2];
+    uint64_t drain;
+};
+
+__device__ __forceinline__ void lt_fail(volatile int* abort_flag, int32_t* status)
+{
+    *abort_flag = 1;
+    record_status(status, SCALE_ERR_TIMEOUT);
+}
+
+__global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, const float* __restrict__ fp,
                                                           const float* __restrict__ reps,
                                                           float* __restrict__ logits)
 {
     using namespace scale_ptx;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t d_full;
+    __shared__ LtBars bars;
     __shared__ uint32_t tmem_slot;
-    __shared__ int64_t s_lo[128], s_hi[128];
-    __shared__ int s_anchor[128];
-    __shared__ int any;
-    const int U = 128 / a.g;  // units per tile
-    const int u_first = unit_lower_bound(a.ut, a.sc_begin);
+    __shared__ volatile int abort_flag;
+    __shared__ int s_hi[kLtSeg * kLtRows], s_anchor[kLtSeg * kLtRows];  // of the segment's units
+    const int U = kLtRows / a.g;  // units per tile
     const int u_end = unit_lower_bound(a.ut, a.sc_end);
-    const int u0 = u_first + static_cast<int>(blockIdx.x) * U;
+    const int u0 = unit_lower_bound(a.ut, a.sc_begin) + static_cast<int>(blockIdx.x) * seg * U;
     if (u0 >= u_end) return;
-    const int n_u = (u_end - u0 < U) ? u_end - u0 : U;
-    const int rows = n_u * a.g;
+    const int n_u = (u_end - u0 < seg * U) ? u_end - u0 : seg * U;
     const int j = blockIdx.z;
     const int64_t b0 = static_cast<int64_t>(blockIdx.y) * 128;
     const int D = a.Hq * kHeadDim;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // The tile is needed only if some unit's candidate range meets [b0, b0 + 128).
-    if (tid == 0) any = 0;
-    __syncthreads();
-    if (tid < n_u) {
-        int64_t s, e, lo, hi;
-        int anc;
-        unit_range(a.ut, u0 + tid, &anc, &s, &e);
+    // The candidates [lo, hi(u)) of the units grow with u: the tiles before the
+    // first unit with a candidate in [b0, b0 + 128) have nothing to do here.
+    int64_t s, e, lo, hi;
+    int anc;
+    unit_range(a.ut, u0 + n_u - 1, &anc, &s, &e);
+    cand_range(a, s, &lo, &hi);
+    if (hi <= b0 || lo >= b0 + 128 || lo >= hi) return;
+    for (int i = tid; i < n_u; i += kLtThreads) {
+        unit_range(a.ut, u0 + i, &anc, &s, &e);
         cand_range(a, s, &lo, &hi);
-        s_lo[tid] = lo;
-        s_hi[tid] = hi;
-        s_anchor[tid] = anc;
-        if (lo < hi && lo < b0 + 128 && hi > b0) atomicOr(&any, 1);
+        s_hi[i] = static_cast<int>(hi);
+        s_anchor[i] = anc;
     }
-    __syncthreads();
-    if (!any) return;
-
     uint8_t* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
-    uint8_t* abuf = smem;                // A parts 0..2
-    uint8_t* bbuf = smem + 3 * kLtPart;  // B parts 0..2
-    // 128 rows x 32 float4 per operand; a warp reads one 512-byte row
-    for (int x = tid; x < 128 * 32; x += kLtThreads) {
-        const int r = x >> 5, c = (x & 31) * 4;
-        float4 va = make_float4(0.f, 0.f, 0.f, 0.f), vb = va;
-        if (r < rows) {
-            const int ul = r / a.g, hl = r % a.g;
-            va = *reinterpret_cast<const float4*>(fp + static_cast<int64_t>(s_anchor[ul]) * D +
-                                                  (j * a.g + hl) * kHeadDim + c);
+    uint8_t* bbuf = smem;                 // representatives, three parts
+    uint8_t* abuf = smem + 3 * kLtBPart;  // two buffers of three parts
+    // a warp reads one 512-byte row; eight rows per thread in flight
+    for (int x0 = tid; x0 < 128 * 32; x0 += 8 * kLtThreads) {
+        float4 v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int x = x0 + i * kLtThreads, r = x >> 5, c = (x & 31) * 4;
+            v[i] = x < 128 * 32 && b0 + r < a.nb
+                       ? __ldg(reinterpret_cast<const float4*>(reps + (j * a.nb + b0 + r) * kHeadDim + c))
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        if (b0 + r < a.nb) vb = *reinterpret_cast<const float4*>(reps + (j * a.nb + b0 + r) * kHeadDim + c);
-        put_split4(abuf, r, c, va);
-        put_split4(bbuf, r, c, vb);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int x = x0 + i * kLtThreads;
+            if (x < 128 * 32) put_split4<kLtBPart>(bbuf, x >> 5, (x & 31) * 4, v[i]);
+        }
     }
     fence_proxy_async_smem();
     if (tid == 0) {
-        mbar_init(&d_full, 1);
+        abort_flag = 0;
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&bars.a_full[i], kLtStageThreads);
+            mbar_init(&bars.a_empty[i], 1);
+            mbar_init(&bars.d_full[i], 1);
+            mbar_init(&bars.d_empty[i], 128);
+        }
+        mbar_init(&bars.drain, 1);
         fence_barrier_init();
     }
-    if (warp == 1) {
+    if (warp == 0) {
         tmem_alloc(&tmem_slot, 128);
         tmem_relinquish();
     }
@@ -162,53 +187,109 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, const float
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-
-    if (tid == 0) {
-        const uint32_t idesc = idesc_bf16_f32(128, 128, 0);
-        const uint64_t ad = sdesc_sw128(smem_addr(abuf), 16, 1024);
-        const uint64_t bd = sdesc_sw128(smem_addr(bbuf), 16, 1024);
-        constexpr uint64_t kPartStep = kLtPart >> 4;
-        // (A part, B part): the products a_i b_j with i + j <= 4 (parts from 1)
-        constexpr int kPa[6] = {0, 0, 1, 0, 1, 2};
-        constexpr int kPb[6] = {0, 1, 0, 2, 1, 0};
-#pragma unroll
-        for (int i = 0; i < 6; ++i)
-            mma_ss_k128<kLtHalf>(tmem, ad + kPa[i] * kPartStep, bd + kPb[i] * kPartStep, idesc, i > 0 ? 1u : 0u);
-        mma_commit(&d_full);
+    int first = 0;  // first unit with a candidate here (the last one has)
+    for (int last = n_u - 1; first < last;) {
+        const int mid = (first + last) >> 1;
+        if (s_hi[mid] <= b0) first = mid + 1;
+        else last = mid;
     }
-    bool done = true;
-    if (warp < 4) {
-        // epilogue: thread = row (TMEM lane) warp * 32 + lane
-        done = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&d_full, 0, a.timeout_ns, nullptr));
-        if (done) {
-            tc_fence_after();
-            const uint32_t lane_base = tmem + (static_cast<uint32_t>(warp * 32) << 16);
-            uint32_t zr[128];
+    const int i0 = first / U, n_it = (n_u + U - 1) / U - i0;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ MMA issuer
+        if (lane == 0) {
+            const uint32_t idesc = idesc_bf16_f32(128, kLtRows, 0);
+            const uint64_t bd = sdesc_sw128(smem_addr(bbuf), 16, 1024);
+            const uint64_t ad0 = sdesc_sw128(smem_addr(abuf), 16, 1024);
+            // (A part, B part): the products a_i b_j with i + j <= 4 (parts from 1)
+            constexpr int kPa[6] = {0, 0, 1, 0, 1, 2};
+            constexpr int kPb[6] = {0, 1, 0, 2, 1, 0};
+            bool ok = true;
+            for (int it = 0; it < n_it; ++it) {
+                const int st = it & 1;
+                if (!mbar_wait_bounded(&bars.a_full[st], (it >> 1) & 1, a.timeout_ns, &abort_flag)) { ok = false; break; }
+                if (it >= 2 && !mbar_wait_bounded(&bars.d_empty[st], ((it >> 1) - 1) & 1, a.timeout_ns, &abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const uint64_t ad = ad0 + st * (3 * kLtAPart >> 4);
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc)
-                tmem_ld32(lane_base + cc * 32, *reinterpret_cast<uint32_t(*)[32]>(&zr[cc * 32]));
-            tmem_ld_wait();
-            const int r = warp * 32 + lane;
-            if (r < rows) {
-                const int ul = r / a.g, hl = r % a.g;
-                const int64_t lo = s_lo[ul] > b0 ? s_lo[ul] : b0;
-                const int64_t hi = s_hi[ul] < b0 + 128 ? s_hi[ul] : b0 + 128;
-                float* dst = logits + (static_cast<int64_t>(u0 + ul) * a.Hq + j * a.g + hl) * a.nb + b0;
-                const int c_lo = static_cast<int>(lo - b0), c_hi = static_cast<int>(hi - b0);
-#pragma unroll
-                for (int c = 0; c < 128; ++c)
-                    if (c >= c_lo && c < c_hi) dst[c] = a.sigma * __uint_as_float(zr[c]);
+                for (int i = 0; i < 6; ++i)
+                    mma_ss_k128_ab<kLtBPart / 2, kLtAPart / 2>(tmem + st * kLtRows, bd + kPb[i] * (kLtBPart >> 4),
+                                                               ad + kPa[i] * (kLtAPart >> 4), idesc, i > 0 ? 1u : 0u);
+                mma_commit(&bars.d_full[st]);
+                mma_commit(&bars.a_empty[st]);
             }
-        } else if (lane == 0) {
-            record_status(a.status, SCALE_ERR_TIMEOUT);
+            if (!ok) {
+                lt_fail(&abort_flag, a.status);
+                mma_commit(&bars.drain);
+                mbar_wait_bounded(&bars.drain, 0, a.timeout_ns, nullptr);
+            }
         }
-    } else if (warp == 4 && lane == 0) {
-        // TMEM is freed only after the MMAs completed (bounded)
-        mbar_wait_bounded(&d_full, 0, a.timeout_ns, nullptr);
+    } else if (warp < 5) {
+        // ------------------------------------------------------------ stores
+        const int q = warp & 3;  // TMEM lane quarter this warp may access
+        const uint32_t lane_base = tmem + (static_cast<uint32_t>(q * 32) << 16);
+        const int64_t b = b0 + q * 32 + lane;  // this thread's block
+        const bool in = b >= a.n_sink / a.B;
+        for (int it = 0; it < n_it; ++it) {
+            const int st = it & 1;
+            if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(&bars.d_full[st], (it >> 1) & 1, a.timeout_ns, &abort_flag))) {
+                if (lane == 0) lt_fail(&abort_flag, a.status);
+                break;
+            }
+            tc_fence_after();
+            uint32_t z[kLtRows];
+            tmem_ld32(lane_base + st * kLtRows, *reinterpret_cast<uint32_t(*)[32]>(&z[0]));
+            tmem_ld32(lane_base + st * kLtRows + 32, *reinterpret_cast<uint32_t(*)[32]>(&z[32]));
+            tmem_ld_wait();
+            tc_fence_before();
+            mbar_arrive(&bars.d_empty[st]);
+            int ul = (i0 + it) * U, left = a.g;
+            float* dst = logits + (static_cast<int64_t>(u0 + ul) * a.Hq + j * a.g) * a.nb + b;
+            bool live = in && ul < n_u && b < s_hi[ul];
+#pragma unroll
+            for (int c = 0; c < kLtRows; ++c) {
+                if (live) *dst = a.sigma * __uint_as_float(z[c]);
+                dst += a.nb;
+                if (--left == 0) {  // the next unit's heads
+                    left = a.g;
+                    ++ul;
+                    dst += static_cast<int64_t>(a.Hq - a.g) * a.nb;
+                    live = in && ul < n_u && ul < (i0 + it + 1) * U && b < s_hi[ul];
+                }
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ staging
+        const int t = tid - 160;
+        for (int it = 0; it < n_it; ++it) {
+            const int st = it & 1;
+            constexpr int kPer = kLtRows * 32 / kLtStageThreads;
+            float4 v[kPer];
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int x = t + i * kLtStageThreads, r = x >> 5, c = (x & 31) * 4;
+                const int ul = r / a.g, u = (i0 + it) * U + ul;
+                v[i] = ul < U && u < n_u
+                           ? __ldg(reinterpret_cast<const float4*>(fp + static_cast<int64_t>(s_anchor[u]) * D +
+                                                                   (j * a.g + r - ul * a.g) * kHeadDim + c))
+                           : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+            if (it >= 2 && !mbar_wait_bounded(&bars.a_empty[st], ((it >> 1) - 1) & 1, a.timeout_ns, &abort_flag)) {
+                lt_fail(&abort_flag, a.status);
+                break;
+            }
+#pragma unroll
+            for (int i = 0; i < kPer; ++i) {
+                const int x = t + i * kLtStageThreads;
+                put_split4<kLtAPart>(abuf + st * 3 * kLtAPart, x >> 5, (x & 31) * 4, v[i]);
+            }
+            fence_proxy_async_smem();
+            mbar_arrive(&bars.a_full[st]);
+        }
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 0) {
         tc_fence_after();
         tmem_dealloc(tmem, 128);
     }
@@ -1237,13 +1318,19 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
         if (ef == cudaSuccess) return ef;
         cudaGetLastError();
     }
-    const int upt = 128 / d.g;  // units per logits tile
-    // set on every launch: the attribute belongs to the current device
-    cudaError_t e = cudaFuncSetAttribute(k_logits, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kLtSmem));
+    // Tiles per CTA: as many as leave every SM a CTA, at most kLtSeg.
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    dim3 gl((max_units + upt - 1) / upt, static_cast<unsigned>((d.nb + 127) / 128), d.Hkv);
-    k_logits<<<gl, kLtThreads, kLtSmem, st>>>(a, fingerprints, reps, logits);
+    const int upt = kLtRows / d.g;  // units per logits tile
+    const int tiles = (max_units + upt - 1) / upt;
+    const int64_t ctas = static_cast<int64_t>(tiles) * ((d.nb + 127) / 128) * d.Hkv;
+    const int seg = ctas >= static_cast<int64_t>(kLtSeg) * sms ? kLtSeg : static_cast<int>((ctas + sms - 1) / sms);
+    // set on every launch: the attribute belongs to the current device
+    e = cudaFuncSetAttribute(k_logits, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLtSmem));
+    if (e != cudaSuccess) return e;
+    dim3 gl((tiles + seg - 1) / seg, static_cast<unsigned>((d.nb + 127) / 128), d.Hkv);
+    k_logits<<<gl, kLtThreads, kLtSmem, st>>>(a, seg, fingerprints, reps, logits);
     if (d.nb <= kSortMax && d.Hq <= kFusedMaxHeads && d.k <= kSortMax) {
         // every unit's candidates fit the sort: statistics, vote and top-k in one kernel
         k_select_fused<<<max_units, kTopkThreads, 0, st>>>(a, logits, scores, sel_blocks, sel_count);
