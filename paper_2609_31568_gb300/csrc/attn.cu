@@ -11,8 +11,8 @@
 // visited once (the de-duplication of Sec. V-A3).
 //
 // Design (one CTA per work item = 128 query rows x 2 query heads of one KV head;
-// with an odd number of query heads per KV head the last one of each group
-// runs alone, as a CTA with one query tile):
+// with an odd number of query heads per KV head, 256 rows of the last one of
+// each group):
 //  - D_u is cut into 64-row segments; two segments form a 128-key tile. Each
 //    segment is one TMA box per 64-column half of head_dim, so gathered blocks
 //    land in shared memory in the 128-byte-swizzled K-major layout the tensor
@@ -74,7 +74,9 @@ struct AttnArgs {
     int n_sc;       // sub-chunks in the token range
     int qb_per_sc;     // 128-row query blocks per sub-chunk
     int sc_per_chunk;  // sub-chunks per outer chunk
-    int Hq, Hkv, g, pairs;
+    int Hq, Hkv, g;
+    int odd_blk;       // query blocks per CTA of an odd group's last head, and
+    int odd_per_sc;    // CTAs per sub-chunk and KV head of that head (0: even group)
     int64_t N, nb;
     int B, k, n_sink, n_local;
     float scale_log2;
@@ -187,30 +189,45 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
     // a time share the K/V rows of one or two KV heads of one cluster (a few
     // MB, which L2 keeps); for each KV head the chunk's last query block
     // comes first, which issues the heaviest rows (longest window) first. ----
-    const int per_chunk = a.sc_per_chunk * a.qb_per_sc;  // query blocks of a full chunk
-    const int per_chunk_ctas = per_chunk * a.Hkv * a.pairs;
+    // A work item has two query tiles: two heads of one query block, or, for
+    // the last head of an odd group, odd_blk neighbouring query blocks of a
+    // sub-chunk. ----
+    const int per_sc_ctas = a.qb_per_sc * (a.g / 2) + a.odd_per_sc;  // of one KV head
+    const int per_chunk_ctas = a.sc_per_chunk * per_sc_ctas * a.Hkv;
     const int c = static_cast<int>(blockIdx.x) / per_chunk_ctas;
     const int sc0 = a.sc_begin + c * a.sc_per_chunk;
     const int n_sc = (a.sc_end - sc0 < a.sc_per_chunk) ? a.sc_end - sc0 : a.sc_per_chunk;
     const int n_qb = n_sc * a.qb_per_sc;  // query blocks of this chunk
     int rem = static_cast<int>(blockIdx.x) - c * per_chunk_ctas;
-    const int kvh = rem / (n_qb * a.pairs);
-    rem -= kvh * n_qb * a.pairs;
-    const int qb = rem / a.pairs;
-    const int h0 = kvh * a.g + 2 * (rem - qb * a.pairs);
-    const int nq = (h0 + 1 < (kvh + 1) * a.g) ? 2 : 1;  // query tiles (heads) of this CTA
-    const int idx = n_qb - 1 - qb;
-    if (idx < 0 || kvh >= a.Hkv) return;
-    const int sc = sc0 + idx / a.qb_per_sc;
+    const int kvh = rem / (n_sc * per_sc_ctas);
+    rem -= kvh * n_sc * per_sc_ctas;
+    if (kvh >= a.Hkv) return;
+    const bool rows2 = rem >= n_qb * (a.g / 2);  // query blocks of one head
+    int sc, blk, h0;
+    if (!rows2) {
+        const int qb = rem / (a.g / 2);
+        h0 = kvh * a.g + 2 * (rem - qb * (a.g / 2));
+        const int idx = n_qb - 1 - qb;
+        sc = idx / a.qb_per_sc;
+        blk = idx - sc * a.qb_per_sc;
+    } else {
+        h0 = kvh * a.g + a.g - 1;
+        const int idx = n_sc * a.odd_per_sc - 1 - (rem - n_qb * (a.g / 2));
+        sc = idx / a.odd_per_sc;
+        blk = a.odd_blk * (idx - sc * a.odd_per_sc);
+    }
+    sc += sc0;
     const int u = unit_of_subchunk(a.ut, sc);
     int anchor;
     int64_t s_u, e_u;
     unit_range(a.ut, u, &anchor, &s_u, &e_u);
     const int64_t sc_lo = static_cast<int64_t>(sc) * a.ut.L;
     const int64_t sc_hi = (sc_lo + a.ut.L < e_u) ? sc_lo + a.ut.L : e_u;
-    const int64_t q0 = sc_lo + static_cast<int64_t>(kRows) * (idx % a.qb_per_sc);
+    const int64_t q0 = sc_lo + static_cast<int64_t>(kRows) * blk;
     if (q0 >= sc_hi) return;
-    const int64_t q_end = (q0 + kRows < sc_hi) ? q0 + kRows : sc_hi;
+    const int nq = !rows2 || (a.odd_blk == 2 && q0 + kRows < sc_hi) ? 2 : 1;  // query tiles of this CTA
+    const int64_t q_last = rows2 ? q0 + kRows * nq : q0 + kRows;
+    const int64_t q_end = q_last < sc_hi ? q_last : sc_hi;
     const int64_t W = (s_u - a.n_local > 0) ? s_u - a.n_local : 0;
     const int n_lt = static_cast<int>((q_end - W + 127) / 128);
 
@@ -312,8 +329,8 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             mbar_arrive_expect_tx(&bars.q_full, nq * kTileBytes);
             for (int qt = 0; qt < nq; ++qt)
                 for (int hf = 0; hf < 2; ++hf)
-                    tma_load_3d(smem + kOffQ + qt * kTileBytes + hf * kHalf, &tq, &bars.q_full,
-                                hf * 64, h0 + qt, static_cast<int32_t>(q0));
+                    tma_load_3d(smem + kOffQ + qt * kTileBytes + hf * kHalf, &tq, &bars.q_full, hf * 64,
+                                rows2 ? h0 : h0 + qt, static_cast<int32_t>(rows2 ? q0 + kRows * qt : q0));
             const int32_t prow = u * a.Hkv + kvh;  // packed (unit, KV head) plane
             // Step t (0..T) loads K(t) and V(t - 1) on kv_full[t & 1]; both stages
             // they reuse were last read by MMAs of iteration t - 2 (Q K^T of K(t - 2),
@@ -412,7 +429,9 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         const int qt = warp >> 2;
         const int quarter = warp & 3;
         const int r = quarter * 32 + lane;
-        const int64_t p = q0 + r;
+        const int64_t q0t = rows2 ? q0 + kRows * qt : q0;  // first row and head of this tile
+        const int head = rows2 ? h0 : h0 + qt;
+        const int64_t p = q0t + r;
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint32_t s_addr = lane_base + qt * 256;
         const uint32_t o_addr = s_addr + 128;
@@ -472,7 +491,7 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
                 lim_b = seg[2 * t + 1].y;
             } else {
                 const int64_t kb = W + 128ll * (t - n_dt);
-                if (kb + 127 > q0) {
+                if (kb + 127 > q0t) {
                     const int64_t lim = p - kb + 1;  // keys kb + c with c >= lim are in the future
                     lim_a = lim < 0 ? 0 : (lim > 128 ? 128 : static_cast<int>(lim));
                     lim_b = lim_a - 64;
@@ -553,7 +572,7 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             tc_fence_after();
             const float inv_l = l_run > 0.f ? 1.0f / l_run : 0.f;
             const bool store = p < q_end;
-            uint4* dst = reinterpret_cast<uint4*>(a.out + (p * a.Hq + h0 + qt) * static_cast<int64_t>(kHeadDim));
+            uint4* dst = reinterpret_cast<uint4*>(a.out + (p * a.Hq + head) * static_cast<int64_t>(kHeadDim));
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 uint32_t v[32];
@@ -758,7 +777,17 @@ cudaError_t launch_sparse_prefill(const Derived& d, int mode, int64_t tok_begin,
     a.Hq = d.Hq;
     a.Hkv = d.Hkv;
     a.g = d.g;
-    a.pairs = (d.g + 1) / 2;  // an odd group's last head runs alone
+    // An odd group's last head: two query blocks per CTA once one block per CTA
+    // would not fit the SMs at a time. A CTA with one query tile runs at the
+    // pace of one softmax chain (8,128 rows of 28 heads on 4, a quarter of the
+    // CTAs with one tile: 691 us; all with two: 627 us), but where
+    // SMs are free twice the CTAs are quicker.
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    const int64_t singles = static_cast<int64_t>(a.n_sc) * d.Hkv * a.qb_per_sc * ((d.g + 1) / 2);
+    a.odd_blk = singles > sms ? 2 : 1;
+    a.odd_per_sc = d.g % 2 ? (a.qb_per_sc + a.odd_blk - 1) / a.odd_blk : 0;
     a.N = d.N;
     a.nb = d.nb;
     a.B = d.B;
@@ -786,10 +815,9 @@ cudaError_t launch_sparse_prefill(const Derived& d, int mode, int64_t tok_begin,
             reinterpret_cast<uint4*>(ws + lay.tok_pack_v), slots);
     }
     auto kern = tok ? k_sparse_attn<true> : k_sparse_attn<false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmemBytes));
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
     if (e != cudaSuccess) return e;
-    const int64_t grid = static_cast<int64_t>(a.n_sc) * a.qb_per_sc * d.Hkv * a.pairs;
+    const int64_t grid = static_cast<int64_t>(a.n_sc) * d.Hkv * (a.qb_per_sc * (d.g / 2) + a.odd_per_sc);
     if (grid <= 0 || grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
     kern<<<static_cast<unsigned>(grid), kThreads, kSmemBytes, st>>>(tq, tk, tv, tpk, tpv, a);
     return cudaGetLastError();

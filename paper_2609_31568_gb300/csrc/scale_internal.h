@@ -152,6 +152,7 @@ __device__ __forceinline__ void record_status(int32_t* status, int32_t code)
 }
 
 // ---- launchers (defined in the .cu files) ----
+cudaError_t device_sms(int* sms);  // SMs of the current device
 cudaError_t launch_build_reps(const Derived& d, const void* q, const void* k, const KvPaging& pg,
                               float* reps, float* fingerprints, int32_t* unit_start, int32_t* n_units,
                               uint8_t* ws, cudaStream_t st);

@@ -62,7 +62,6 @@ struct VoteArgs {
     uint64_t timeout_ns;
 };
 
-cudaError_t device_sms(int* sms);  // SMs of the current device
 // CTAs per unit tile of k_key_logits (= partials per head): two per SM, at most
 // one per (128-key tile, KV head) and at most `room`.
 int key_logits_parts(int64_t cand_end, int Hkv, int64_t room);
