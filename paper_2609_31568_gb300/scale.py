@@ -106,6 +106,8 @@ def declared_functions() -> list[str]:
 
 def load() -> ctypes.CDLL:
     global _lib
+    if _lib is not None:  # set once, after its signatures: every call comes through here
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -147,36 +149,40 @@ def load() -> ctypes.CDLL:
             f.argtypes = args
             f.restype = ctypes.c_int
         lib.scale_status_string.restype = ctypes.c_char_p
-        _lib = lib
+        _lib = lib  # the library is complete here
         return lib
 
 
 def _ptr(x) -> int | None:
     """Device or host address of a tensor / array / int (None for None)."""
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or isinstance(x, int):
         return x
-    if hasattr(x, "data_ptr"):
+    data_ptr = getattr(x, "data_ptr", None)
+    if data_ptr is not None:
         if not x.is_contiguous():
             raise ValueError("tensors passed to libscale must be contiguous")
-        return x.data_ptr()
+        return data_ptr()
     if hasattr(x, "ctypes"):
         return x.ctypes.data
     raise TypeError(f"cannot pass {type(x).__name__} as a pointer")
 
 
 def _nbytes(x) -> int:
-    if hasattr(x, "numel"):
-        return x.numel() * x.element_size()
     return int(x.nbytes)
+
+
+_torch = None  # the torch module, once a call has needed its current stream
 
 
 def _stream(stream) -> int | None:
     if stream is None:
-        import torch
+        global _torch
+        if _torch is None:
+            import torch
 
-        return torch.cuda.current_stream().cuda_stream
+            _torch = torch
+        # the handle alone: 0.3 us, against 3 us for a torch.cuda.Stream object
+        return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
