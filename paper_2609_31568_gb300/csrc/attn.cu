@@ -35,6 +35,7 @@
 //    returns.
 #include <cuda_bf16.h>
 
+#include "launch.cuh"
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
 #include "tma_host.h"
@@ -181,6 +182,21 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
     __shared__ int s_nseg;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        abort_flag = 0;
+        mbar_init(&bars.q_full, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&bars.kv_full[i], 1);
+            mbar_init(&bars.s_full[i][0], 1);
+            mbar_init(&bars.s_full[i][1], 1);
+            mbar_init(&bars.p_full[i], 128);
+        }
+        mbar_init(&bars.o_full, 1);
+        mbar_init(&bars.drain, 1);
+        fence_barrier_init();
+    }
+    pdl_enter();
 
     // ---- work item: a 128-row query block of one sub-chunk and a pair of
     // query heads. The grid holds exactly the blocks of the sub-chunks in
@@ -233,21 +249,7 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
 
     uint8_t* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     int2* seg = reinterpret_cast<int2*>(smem + kOffSeg);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    if (tid == 0) {
-        abort_flag = 0;
-        mbar_init(&bars.q_full, 1);
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&bars.kv_full[i], 1);
-            mbar_init(&bars.s_full[i][0], 1);
-            mbar_init(&bars.s_full[i][1], 1);
-            mbar_init(&bars.p_full[i], 128);
-        }
-        mbar_init(&bars.o_full, 1);
-        mbar_init(&bars.drain, 1);
-        fence_barrier_init();
-    }
     if (warp == 9) {
         tmem_alloc(&tmem_slot, 512);
         tmem_relinquish();
@@ -615,6 +617,7 @@ __global__ void __launch_bounds__(kListThreads) k_tok_lists(Units ut, int sc_beg
                                                             int slots)
 {
     __shared__ int s_warp[kListThreads / 32];
+    pdl_enter();
     const int u = unit_lower_bound(ut, sc_begin) + static_cast<int>(blockIdx.x);
     if (u >= unit_lower_bound(ut, sc_end)) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -685,6 +688,7 @@ __global__ void __launch_bounds__(256) k_tok_pack(Units ut, int sc_begin, int sc
                                                   const uint4* __restrict__ kin, const uint4* __restrict__ vin,
                                                   uint4* __restrict__ kout, uint4* __restrict__ vout, int slots)
 {
+    pdl_enter();
     const int u = unit_lower_bound(ut, sc_begin) + static_cast<int>(blockIdx.x);
     if (u >= unit_lower_bound(ut, sc_end)) return;
     const int kvh = blockIdx.y;
@@ -807,20 +811,21 @@ cudaError_t launch_sparse_prefill(const Derived& d, int mode, int64_t tok_begin,
     if (tok) {
         int32_t* list = reinterpret_cast<int32_t*>(ws + lay.tok_list);
         int32_t* cnt = const_cast<int32_t*>(a.tok_count);
-        k_tok_lists<<<a.n_sc, kListThreads, 0, st>>>(a.ut, a.sc_begin, a.sc_end, d.n_sink, d.n_local, d.k, sel_blocks,
-                                           sel_count, list, cnt, slots);
-        k_tok_pack<<<dim3(a.n_sc, d.Hkv, (slots + kPackSlots - 1) / kPackSlots), 256, 0, st>>>(
-            a.ut, a.sc_begin, a.sc_end, d.Hkv, pg, list, cnt, static_cast<const uint4*>(k),
-            static_cast<const uint4*>(v), reinterpret_cast<uint4*>(ws + lay.tok_pack_k),
-            reinterpret_cast<uint4*>(ws + lay.tok_pack_v), slots);
+        e = launch_after(st, dim3(a.n_sc), kListThreads, 0, 1, k_tok_lists, a.ut, a.sc_begin, a.sc_end, d.n_sink,
+                         d.n_local, d.k, sel_blocks, sel_count, list, cnt, slots);
+        if (e == cudaSuccess)
+            e = launch_after(st, dim3(a.n_sc, d.Hkv, (slots + kPackSlots - 1) / kPackSlots), 256, 0, 1, k_tok_pack, a.ut,
+                             a.sc_begin, a.sc_end, d.Hkv, pg, list, cnt, static_cast<const uint4*>(k),
+                             static_cast<const uint4*>(v), reinterpret_cast<uint4*>(ws + lay.tok_pack_k),
+                             reinterpret_cast<uint4*>(ws + lay.tok_pack_v), slots);
+        if (e != cudaSuccess) return e;
     }
     auto kern = tok ? k_sparse_attn<true> : k_sparse_attn<false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
     if (e != cudaSuccess) return e;
     const int64_t grid = static_cast<int64_t>(a.n_sc) * d.Hkv * (a.qb_per_sc * (d.g / 2) + a.odd_per_sc);
     if (grid <= 0 || grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
-    kern<<<static_cast<unsigned>(grid), kThreads, kSmemBytes, st>>>(tq, tk, tv, tpk, tpv, a);
-    return cudaGetLastError();
+    return launch_after(st, dim3(static_cast<unsigned>(grid)), kThreads, kSmemBytes, 1, kern, tq, tk, tv, tpk, tpv, a);
 }
 
 cudaError_t launch_wait_selftest(uint8_t* ws, uint64_t timeout_ns, cudaStream_t st)

@@ -23,6 +23,7 @@
 
 #include <cmath>
 
+#include "launch.cuh"
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
 #include "score.cuh"
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const 
     __shared__ float2 s_ml[kDecWarps][G];
     __shared__ float s_w[G][kDecMaxSplits];
     __shared__ int s_last;
+    pdl_enter();
     const int j = blockIdx.x, split = blockIdx.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int half = lane >> 4, c = lane & 15;
@@ -326,10 +328,9 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const 
 template <int G>
 cudaError_t run_dec_attn(const DecArgs& a, const void* q, const void* k, const void* v, void* out, cudaStream_t st)
 {
-    k_dec_attn<G><<<dim3(a.Hkv, a.splits), kDecThreads, 0, st>>>(
-        a, static_cast<const __nv_bfloat16*>(q), static_cast<const uint4*>(k), static_cast<const uint4*>(v),
-        static_cast<__nv_bfloat16*>(out));
-    return cudaGetLastError();
+    return launch_after(st, dim3(a.Hkv, a.splits), kDecThreads, 0, 1, k_dec_attn<G>, a,
+                        static_cast<const __nv_bfloat16*>(q), static_cast<const uint4*>(k),
+                        static_cast<const uint4*>(v), static_cast<__nv_bfloat16*>(out));
 }
 
 // Chunks of 64 keys that the workspace holds a (max, sum) pair for.

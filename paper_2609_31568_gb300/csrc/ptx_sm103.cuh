@@ -146,6 +146,32 @@ __device__ __forceinline__ void named_barrier(uint32_t id, uint32_t count)
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// ------------------------------------------------------------------ dependent launches
+
+// A kernel launched by launch_after() may start while the kernel before it on
+// the stream still runs: pdl_wait() returns once that one has completed and its
+// writes are visible. Every thread calls it before any access to global memory,
+// and no thread returns before it, so a kernel never completes before those
+// ahead of it.
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// Allow the next kernel's CTAs on the SMs that this kernel leaves free, once
+// every CTA of it has called this (or has exited).
+__device__ __forceinline__ void pdl_trigger()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// pdl_wait, then pdl_trigger: one dependent kernel waits at a time.
+__device__ __forceinline__ void pdl_enter()
+{
+    pdl_wait();
+    pdl_trigger();
+}
+
 // ------------------------------------------------------------------ clusters
 
 __device__ __forceinline__ uint32_t cluster_ctarank()

@@ -10,6 +10,8 @@
 // with the same per-element arithmetic as over the whole sequence.
 #include <cuda_bf16.h>
 
+#include "launch.cuh"
+#include "ptx_sm103.cuh"
 #include "scale_internal.h"
 
 namespace scale {
@@ -267,6 +269,7 @@ __global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __rest
 {
     __shared__ int sh[40];
     __shared__ int last;
+    scale_ptx::pdl_enter();
     const float* fp = args.fp;
     const float* ss_part = args.ss_part;
     const int groups = args.fp_groups, D = args.D8 * 8, M = args.M, S_max = args.S_max, per_outer = args.per_outer;
@@ -314,6 +317,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_step_a(const StepArgs a)
     __shared__ float4 part[kStepThreads * 2];
     __shared__ float wsum[8];
     __shared__ int sh[40];
+    scale_ptx::pdl_enter();
     int x = blockIdx.x;
     if (x == 0) {
         if (threadIdx.x == 0) *a.ticket = 0;
@@ -391,13 +395,13 @@ cudaError_t launch_build_reps_range(const Derived& d, const void* q, const void*
     const int64_t rep_ctas = reps && b1 > b0 ? (b1 - b0) * a.splits : 0;
     const int64_t grid = 1 + static_cast<int64_t>(a.nm) * a.fp_groups + rep_ctas;
     if (grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
-    k_step_a<<<static_cast<unsigned>(grid), kStepThreads, 0, st>>>(a);
-    if (d.S_max > 1 && d.theta > -1.0f) {
+    cudaError_t e = launch_after(st, dim3(static_cast<unsigned>(grid)), kStepThreads, 0, 1, k_step_a, a);
+    if (e == cudaSuccess && d.S_max > 1 && d.theta > -1.0f) {
         // a warp per cosine, and enough threads to compact the anchors
         const int warps = d.S_max - 1 < 8 ? 8 : d.S_max - 1 < 16 ? d.S_max - 1 : 16;
-        k_gram<<<static_cast<unsigned>(a.nm), 32 * warps, 0, st>>>(a, gram);
+        e = launch_after(st, dim3(static_cast<unsigned>(a.nm)), 32 * warps, 0, 1, k_gram, a, gram);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 cudaError_t launch_build_reps(const Derived& d, const void* q, const void* k, const KvPaging& pg,

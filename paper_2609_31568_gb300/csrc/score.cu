@@ -14,6 +14,7 @@
 // against 2,048 bytes per token and unit for 32 query heads on 8 KV heads.
 #include <cuda_bf16.h>
 
+#include "launch.cuh"
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
 #include "score.cuh"
@@ -140,6 +141,7 @@ k_key_logits(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUt
     __shared__ volatile int abort_flag;
     __shared__ int s_W[US];
     __shared__ float s_max[4][kLgCols], s_sum[4][kLgCols];
+    pdl_enter();
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
@@ -494,6 +496,7 @@ __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
     __shared__ float2 s_stat[kVtMaxHeads];
     __shared__ int s_scan[kVtWarps], s_gt[kVtWarps], s_eq[kVtWarps];
     __shared__ int s_digit, s_need;
+    pdl_trigger();  // launched plainly: what is before it has completed
     if (a.gate && !*a.gate) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
@@ -712,8 +715,7 @@ cudaError_t run_key_logits(const CUtensorMap& tf, const CUtensorMap& tk, const K
     if (e != cudaSuccess) return e;
     constexpr int US = kLgCols / G;
     const dim3 grid(static_cast<unsigned>(a.n_part), static_cast<unsigned>((max_units + US - 1) / US));
-    k_key_logits<G, PARTS><<<grid, kLgThreads, kLgSmem, st>>>(tf, tk, a);
-    return cudaGetLastError();
+    return launch_after(st, grid, kLgThreads, kLgSmem, 1, k_key_logits<G, PARTS>, tf, tk, a);
 }
 
 template <int PARTS>
@@ -781,10 +783,9 @@ cudaError_t launch_vote_topk(const VoteArgs& a, cudaStream_t st)
     for (int grid = sms < kVoteMaxCtas ? sms : kVoteMaxCtas;; grid /= 2) {
         e = cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_vote_topk), dim3(static_cast<unsigned>(grid)),
                                         dim3(kVtThreads), params, kVtSmem, st);
-        if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1) break;
-        cudaGetLastError();
+        if (e != cudaSuccess) cudaGetLastError();  // reported by the return value
+        if (e != cudaErrorCooperativeLaunchTooLarge || grid == 1) return e;
     }
-    return e;
 }
 
 }  // namespace scale

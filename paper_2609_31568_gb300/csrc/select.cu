@@ -19,6 +19,7 @@
 
 #include <cmath>
 
+#include "launch.cuh"
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
 
@@ -125,6 +126,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
     __shared__ int s_hi[kLtSeg * kLtRows], s_anchor[kLtSeg * kLtRows];  // of the segment's units
+    pdl_enter();
     const int U = kLtRows / a.g;  // units per tile
     const int u_end = unit_lower_bound(a.ut, a.sc_end);
     const int u0 = unit_lower_bound(a.ut, a.sc_begin) + static_cast<int>(blockIdx.x) * seg * U;
@@ -692,6 +694,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
     __shared__ uint32_t sk[kSortMax];
     __shared__ TopkShared sh;
+    scale_ptx::pdl_enter();
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
     const int u_end = unit_lower_bound(a.ut, a.sc_end);
     const int u = u_first + blockIdx.x;
@@ -823,6 +826,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     __shared__ float2 s_part[kFewCtas][kFusedMaxHeads];
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
     __shared__ TopkShared sh;
+    pdl_enter();
     const int u = unit_lower_bound(a.ut, a.sc_begin) + static_cast<int>(blockIdx.y);
     if (u >= unit_lower_bound(a.ut, a.sc_end)) return;  // the whole cluster
     int anc;
@@ -940,19 +944,8 @@ cudaError_t run_select_few(const SelArgs& a, const FewPlan& p, int max_units, co
                                          static_cast<int>(p.smem));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_few<G>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(kFewCtas, static_cast<unsigned>(max_units));
-    cfg.blockDim = dim3(kFewThreads);
-    cfg.dynamicSmemBytes = p.smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = kFewCtas;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_select_few<G>, a, fp, reps, p.stride, scores, sel, sel_count);
+    return launch_after(st, dim3(kFewCtas, static_cast<unsigned>(max_units)), kFewThreads, p.smem, kFewCtas,
+                        k_select_few<G>, a, fp, reps, p.stride, scores, sel, sel_count);
 }
 
 cudaError_t launch_select_few(const Derived& d, const SelArgs& a, const FewPlan& p, int max_units, const float* fp,
@@ -1316,7 +1309,6 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
         const cudaError_t ef = launch_select_few(d, a, few, max_units, fingerprints, reps, sel_scores, sel_blocks,
                                                  sel_count, st);
         if (ef == cudaSuccess) return ef;
-        cudaGetLastError();
     }
     // Tiles per CTA: as many as leave every SM a CTA, at most kLtSeg.
     int sms = 0;
@@ -1330,11 +1322,12 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
     e = cudaFuncSetAttribute(k_logits, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kLtSmem));
     if (e != cudaSuccess) return e;
     dim3 gl((tiles + seg - 1) / seg, static_cast<unsigned>((d.nb + 127) / 128), d.Hkv);
-    k_logits<<<gl, kLtThreads, kLtSmem, st>>>(a, seg, fingerprints, reps, logits);
+    e = launch_after(st, gl, kLtThreads, kLtSmem, 1, k_logits, a, seg, fingerprints, reps, logits);
+    if (e != cudaSuccess) return e;
     if (d.nb <= kSortMax && d.Hq <= kFusedMaxHeads && d.k <= kSortMax) {
         // every unit's candidates fit the sort: statistics, vote and top-k in one kernel
-        k_select_fused<<<max_units, kTopkThreads, 0, st>>>(a, logits, scores, sel_blocks, sel_count);
-        return cudaGetLastError();
+        return launch_after(st, dim3(max_units), kTopkThreads, 0, 1, k_select_fused, a, logits, scores, sel_blocks,
+                            sel_count);
     }
     const int64_t rows = static_cast<int64_t>(max_units) * d.Hq;
     k_stats<<<static_cast<unsigned>((rows + 7) / 8), 256, 0, st>>>(a, logits, stats);

@@ -36,6 +36,7 @@
 // is bounded; on expiry the kernel records SCALE_ERR_TIMEOUT and drains.
 #include <cuda_bf16.h>
 
+#include "launch.cuh"
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
 #include "score.cuh"
@@ -671,6 +672,7 @@ k_tok_score_s(const __grid_constant__ CUtensorMap tfs, const __grid_constant__ C
 __global__ void __launch_bounds__(128) k_tok_split(TokArgs a, const float* __restrict__ fp,
                                                    __nv_bfloat16* __restrict__ parts, int M)
 {
+    pdl_enter();
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
     const int u_end = unit_lower_bound(a.ut, a.sc_end);
     const int u = u_first + static_cast<int>(blockIdx.x) / a.Hq;
@@ -822,9 +824,10 @@ cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, 
         !scale_host::make_token_major_map(&tk, k, kHeadDim, d.Hkv, pg.page_table ? pg.pool_rows : d.N, 64, 64))
         return cudaErrorInvalidValue;
 
-    k_tok_split<<<static_cast<unsigned>(max_units) * d.Hq, 128, 0, st>>>(a, fingerprints, parts, static_cast<int>(d.M));
+    cudaError_t e = launch_after(st, dim3(static_cast<unsigned>(max_units) * d.Hq), 128, 0, 1, k_tok_split, a,
+                                 fingerprints, parts, static_cast<int>(d.M));
+    if (e != cudaSuccess) return e;
     const int64_t rows = static_cast<int64_t>(max_units) * d.Hq;
-    cudaError_t e = cudaSuccess;
     // Few units (every call of the Algorithm 2 loop): one read of K with a plane
     // of logits per unit, and the vote and the top-k in one kernel (score.cu).
     // The planes live in the space of the packed rows, which the attention call
