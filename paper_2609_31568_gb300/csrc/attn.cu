@@ -100,6 +100,32 @@ struct Barriers {
     uint64_t drain;
 };
 
+// (unit, its first sub-chunk, one past its last) of the unit that contains
+// sub-chunk sc, by the whole warp: 32 starts are compared at a time, so a table
+// of up to 32 units costs one round of loads (a thread's binary search took
+// five, 2,400 cycles at the start of every CTA).
+__device__ __forceinline__ int3 warp_unit_of_subchunk(const Units& t, int sc)
+{
+    if (t.per_subchunk) return make_int3(sc, sc, sc + 1);
+    const int lane = threadIdx.x & 31;
+    int v = t.unit_start[lane < t.M ? lane : t.M];
+    int lo = 0, n = *t.n_units;
+    while (n > 32) {
+        const int step = (n + 31) / 32, i = lane * step;
+        v = i < n ? t.unit_start[lo + i] : 0x7FFFFFFF;
+        const int k = __popc(__ballot_sync(0xFFFFFFFFu, v <= sc)) - 1;
+        lo += (k > 0 ? k : 0) * step;
+        n -= (k > 0 ? k : 0) * step;
+        n = n < step ? n : step;
+        v = t.unit_start[lo + lane < t.M ? lo + lane : t.M];
+    }
+    int k = __popc(__ballot_sync(0xFFFFFFFFu, lane < n && v <= sc)) - 1;
+    k = k > 0 ? k : 0;
+    const int first = __shfl_sync(0xFFFFFFFFu, v, k);
+    const int end = k < 31 ? __shfl_sync(0xFFFFFFFFu, v, k + 1) : t.unit_start[lo + 32];
+    return make_int3(lo + k, first, end);
+}
+
 __device__ __forceinline__ void fail(volatile int* abort_flag, int32_t* status)
 {
     *abort_flag = 1;
@@ -196,6 +222,16 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         mbar_init(&bars.drain, 1);
         fence_barrier_init();
     }
+    if (tid == 256) {  // the descriptors are parameters: fetched before the wait
+        tma_prefetch_desc(&tq);
+        tma_prefetch_desc(&tk);
+        tma_prefetch_desc(&tv);
+        if (TOK) {
+            tma_prefetch_desc(&tpk);
+            tma_prefetch_desc(&tpv);
+        }
+    }
+    __syncthreads();
     pdl_enter();
 
     // ---- work item: a 128-row query block of one sub-chunk and a pair of
@@ -233,10 +269,10 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         blk = a.odd_blk * (idx - sc * a.odd_per_sc);
     }
     sc += sc0;
-    const int u = unit_of_subchunk(a.ut, sc);
-    int anchor;
-    int64_t s_u, e_u;
-    unit_range(a.ut, u, &anchor, &s_u, &e_u);
+    const int3 unit = warp_unit_of_subchunk(a.ut, sc);
+    const int u = unit.x;
+    const int64_t s_u = static_cast<int64_t>(unit.y) * a.ut.L;
+    const int64_t e_u = static_cast<int64_t>(unit.z) * a.ut.L < a.N ? static_cast<int64_t>(unit.z) * a.ut.L : a.N;
     const int64_t sc_lo = static_cast<int64_t>(sc) * a.ut.L;
     const int64_t sc_hi = (sc_lo + a.ut.L < e_u) ? sc_lo + a.ut.L : e_u;
     const int64_t q0 = sc_lo + static_cast<int64_t>(kRows) * blk;
@@ -254,6 +290,14 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         tmem_alloc(&tmem_slot, 512);
         tmem_relinquish();
     }
+    if (warp == 8 && lane == 0) {
+        // the query tiles are on their way while the distant list is built
+        mbar_arrive_expect_tx(&bars.q_full, nq * kTileBytes);
+        for (int qt = 0; qt < nq; ++qt)
+            for (int hf = 0; hf < 2; ++hf)
+                tma_load_3d(smem + kOffQ + qt * kTileBytes + hf * kHalf, &tq, &bars.q_full, hf * 64,
+                            rows2 ? h0 : h0 + qt, static_cast<int32_t>(rows2 ? q0 + kRows * qt : q0));
+    }
     if (TOK && warp == 8) {
         if (lane == 0) {
             int n = a.tok_count[u];
@@ -262,7 +306,14 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         }
     } else if (warp == 8) {
         // Distant segments: the sinks, then each selected block clipped to
-        // [n_sink, W); 64 rows at most per segment.
+        // [n_sink, W); 64 rows at most per segment. The count and the first
+        // 32 kSelAhead blocks are loaded together.
+        constexpr int kSelAhead = 4;
+        const int32_t* sl = a.sel + static_cast<int64_t>(u) * a.k;
+        int32_t ahead[kSelAhead];
+#pragma unroll
+        for (int i = 0; i < kSelAhead; ++i) ahead[i] = lane + 32 * i < a.k ? sl[lane + 32 * i] : -1;
+        int cnt = a.sel_count[u];
         const int64_t sink_end = a.n_sink < W ? a.n_sink : W;
         const int n_sink_seg = static_cast<int>((sink_end + 63) / 64);
         for (int i = lane; i < n_sink_seg; i += 32) {
@@ -270,17 +321,27 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             seg[i] = make_int2(static_cast<int>(t0), static_cast<int>(sink_end - t0 < 64 ? sink_end - t0 : 64));
         }
         int base = n_sink_seg;
-        int cnt = a.sel_count[u];
         cnt = cnt < 0 ? 0 : (cnt > a.k ? a.k : cnt);
-        const int32_t* sl = a.sel + static_cast<int64_t>(u) * a.k;
         bool overflow = false;
+        int before = -1;  // the entry ahead of this group of 32
         for (int c0 = 0; c0 < cnt; c0 += 32) {
             const int i = c0 + lane;
             int nseg = 0;
             int64_t lo = 0, hi = 0;
+            int32_t entry = -1;
+            if (c0 < 32 * kSelAhead) {
+#pragma unroll
+                for (int x = 0; x < kSelAhead; ++x)
+                    if (c0 == 32 * x) entry = ahead[x];
+            } else if (i < cnt) {
+                entry = sl[i];
+            }
+            int32_t above = __shfl_up_sync(0xFFFFFFFFu, entry, 1);
+            if (lane == 0) above = before;
+            before = __shfl_sync(0xFFFFFFFFu, entry, 31);
             if (i < cnt) {
-                const int64_t b = sl[i];
-                const int64_t prev = i > 0 ? sl[i - 1] : -1;
+                const int64_t b = entry;
+                const int64_t prev = above;
                 if (b >= 0 && b < a.nb && b > prev) {
                     lo = b * a.B > a.n_sink ? b * a.B : a.n_sink;
                     hi = (b + 1) * a.B < W ? (b + 1) * a.B : W;
@@ -321,18 +382,6 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
     if (warp == 8) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            tma_prefetch_desc(&tq);
-            tma_prefetch_desc(&tk);
-            tma_prefetch_desc(&tv);
-            if (TOK) {
-                tma_prefetch_desc(&tpk);
-                tma_prefetch_desc(&tpv);
-            }
-            mbar_arrive_expect_tx(&bars.q_full, nq * kTileBytes);
-            for (int qt = 0; qt < nq; ++qt)
-                for (int hf = 0; hf < 2; ++hf)
-                    tma_load_3d(smem + kOffQ + qt * kTileBytes + hf * kHalf, &tq, &bars.q_full, hf * 64,
-                                rows2 ? h0 : h0 + qt, static_cast<int32_t>(rows2 ? q0 + kRows * qt : q0));
             const int32_t prow = u * a.Hkv + kvh;  // packed (unit, KV head) plane
             // Step t (0..T) loads K(t) and V(t - 1) on kv_full[t & 1]; both stages
             // they reuse were last read by MMAs of iteration t - 2 (Q K^T of K(t - 2),
@@ -437,6 +486,7 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint32_t s_addr = lane_base + qt * 256;
         const uint32_t o_addr = s_addr + 128;
+        const int n_packed = TOK ? s_nseg : 0;
         float m_run = -INFINITY, l_run = 0.f;
         bool ok = true;
         // S row of tile t: four 32-column TMEM loads in flight, one wait, then
@@ -483,7 +533,7 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             // Mask limits of tile t (128: nothing masked).
             int lim_a = 128, lim_b = 128;
             if (TOK && t < n_dt) {
-                const int lim = s_nseg - 128 * t;  // packed rows past the list are zero padding
+                const int lim = n_packed - 128 * t;  // packed rows past the list are zero padding
                 if (lim < 128) {
                     lim_a = lim < 0 ? 0 : lim;
                     lim_b = lim_a - 64;
@@ -573,22 +623,33 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         if (go) {
             tc_fence_after();
             const float inv_l = l_run > 0.f ? 1.0f / l_run : 0.f;
-            const bool store = p < q_end;
-            uint4* dst = reinterpret_cast<uint4*>(a.out + (p * a.Hq + head) * static_cast<int64_t>(kHeadDim));
+            // Every MMA is done, so the tile's Q rows in shared memory are free: a
+            // warp stages its 32 output rows there (16-byte chunk c of row x at
+            // chunk c ^ (x % 16), free of bank conflicts both ways) and stores two
+            // whole rows at a time. A thread storing its own row wrote 32 rows 8 KB
+            // apart per instruction: 5,200 cycles at the end of every CTA.
+            uint32_t v[128];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                uint32_t v[32];
-                tmem_ld32(o_addr + c * 32, v);
-                tmem_ld_wait();
-                if (store) {
+            for (int c = 0; c < 4; ++c) tmem_ld32(o_addr + c * 32, *reinterpret_cast<uint32_t(*)[32]>(&v[c * 32]));
+            tmem_ld_wait();
+            uint8_t* rows = smem + kOffQ + qt * kTileBytes + quarter * 32 * 256;
 #pragma unroll
-                    for (int i = 0; i < 4; ++i)
-                        dst[c * 4 + i] = make_uint4(
-                            pack_bf16x2(__uint_as_float(v[8 * i + 0]) * inv_l, __uint_as_float(v[8 * i + 1]) * inv_l),
-                            pack_bf16x2(__uint_as_float(v[8 * i + 2]) * inv_l, __uint_as_float(v[8 * i + 3]) * inv_l),
-                            pack_bf16x2(__uint_as_float(v[8 * i + 4]) * inv_l, __uint_as_float(v[8 * i + 5]) * inv_l),
-                            pack_bf16x2(__uint_as_float(v[8 * i + 6]) * inv_l, __uint_as_float(v[8 * i + 7]) * inv_l));
-                }
+            for (int c = 0; c < 16; ++c) {
+                uint32_t w[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    w[i] = pack_bf16x2(__uint_as_float(v[8 * c + 2 * i]) * inv_l, __uint_as_float(v[8 * c + 2 * i + 1]) * inv_l);
+                *reinterpret_cast<uint4*>(rows + lane * 256 + ((c ^ (lane & 15)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            __syncwarp();
+            const int c = lane & 15;
+            const int64_t p0 = q0t + quarter * 32;
+            uint4* dst = reinterpret_cast<uint4*>(a.out + (p0 * a.Hq + head) * static_cast<int64_t>(kHeadDim)) + c;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                const int x = 2 * i + (lane >> 4);
+                const uint4 w = *reinterpret_cast<const uint4*>(rows + x * 256 + ((c ^ (x & 15)) << 4));
+                if (p0 + x < q_end) dst[static_cast<int64_t>(x) * a.Hq * (kHeadDim / 8)] = w;
             }
         } else {
             fail(&abort_flag, a.status);
