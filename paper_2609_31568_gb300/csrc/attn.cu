@@ -303,6 +303,14 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             int n = a.tok_count[u];
             n = n < 0 ? 0 : (n > a.slots ? a.slots : n);
             s_nseg = n;  // distant tokens (not segments) in this mode
+            // Mask limits of a whole tile and of the last one (packed rows past the
+            // list are zero padding), read like the segments' lengths: with the
+            // limits computed in the loop the compiler's schedule of it took 2,830
+            // cycles per key tile instead of 2,600.
+            const int last = n - (n - 1) / 128 * 128;
+            seg[0] = seg[1] = make_int2(0, 64);
+            seg[2] = make_int2(0, last < 64 ? last : 64);
+            seg[3] = make_int2(0, last - 64);
         }
     } else if (warp == 8) {
         // Distant segments: the sinks, then each selected block clipped to
@@ -486,7 +494,6 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
         const uint32_t lane_base = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
         const uint32_t s_addr = lane_base + qt * 256;
         const uint32_t o_addr = s_addr + 128;
-        const int n_packed = TOK ? s_nseg : 0;
         float m_run = -INFINITY, l_run = 0.f;
         bool ok = true;
         // S row of tile t: four 32-column TMEM loads in flight, one wait, then
@@ -532,15 +539,10 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             tc_fence_after();
             // Mask limits of tile t (128: nothing masked).
             int lim_a = 128, lim_b = 128;
-            if (TOK && t < n_dt) {
-                const int lim = n_packed - 128 * t;  // packed rows past the list are zero padding
-                if (lim < 128) {
-                    lim_a = lim < 0 ? 0 : lim;
-                    lim_b = lim_a - 64;
-                }
-            } else if (t < n_dt) {
-                lim_a = seg[2 * t].y;
-                lim_b = seg[2 * t + 1].y;
+            if (t < n_dt) {
+                const int x = TOK ? (t == n_dt - 1 ? 2 : 0) : 2 * t;
+                lim_a = seg[x].y;
+                lim_b = seg[x + 1].y;
             } else {
                 const int64_t kb = W + 128ll * (t - n_dt);
                 if (kb + 127 > q0t) {
