@@ -58,25 +58,29 @@ __device__ __forceinline__ void cand_range(const SelArgs& a, int64_t s, int64_t*
 // a_i b_j with i + j <= 4 are exact in fp32 and are accumulated in fp32 in TMEM;
 // the three dropped ones are below 2^-24 of |a| |b|. Only candidate blocks of
 // each row's unit are written. Warp 0 lane 0 issues the MMAs (two accumulators
-// of 64 columns), warps 1-4 store, warps 5-12 load and split the next tile: the
+// of 64 columns), warps 1-8 store, warps 9-16 load and split the next tile: the
 // three overlap, and what bounds the kernel is the staging of a tile. 256
-// units x 4,096 blocks x 32 heads: 81 us (one CTA per tile, staging both
+// units x 4,096 blocks x 32 heads: 63 us (one CTA per tile, staging both
 // operands each time and nothing overlapped: 185 us).
 constexpr int kLtStageThreads = 256;
-constexpr int kLtThreads = 32 + 128 + kLtStageThreads;
+constexpr int kLtStoreThreads = 256;
+constexpr int kLtThreads = 32 + kLtStoreThreads + kLtStageThreads;
 constexpr int kLtRows = 64;                        // (unit, head) rows of a tile
+constexpr int kLtWarpRows = 32;                    // of which a storing warp takes half
 constexpr int kLtSeg = 8;                          // most tiles of a CTA
 constexpr uint32_t kLtBPart = 128 * 128 * 2;       // one bf16 part of the representatives
 constexpr uint32_t kLtAPart = kLtRows * 128 * 2;   // one bf16 part of a tile's rows
 constexpr uint32_t kLtSmem = 3 * kLtBPart + 2 * 3 * kLtAPart + 1024;
 static_assert(kLtSmem + kLtSeg * kLtRows * 8 + 1024 <= 227 * 1024, "logits shared memory");
 
-__device__ __forceinline__ void split_bf16x3(float x, __nv_bfloat16& p1, __nv_bfloat16& p2, __nv_bfloat16& p3)
+// Two fp32 values as three packed bf16 pairs, x1 + x2 + x3 = x for each.
+__device__ __forceinline__ void split_pair(float x, float y, uint32_t (&p)[3])
 {
-    p1 = __float2bfloat16_rn(x);
-    const float r1 = x - __bfloat162float(p1);
-    p2 = __float2bfloat16_rn(r1);
-    p3 = __float2bfloat16_rn(r1 - __bfloat162float(p2));
+    p[0] = scale_ptx::pack_bf16x2(x, y);
+    x -= __uint_as_float(p[0] << 16);
+    y -= __uint_as_float(p[0] & 0xFFFF0000u);
+    p[1] = scale_ptx::pack_bf16x2(x, y);
+    p[2] = scale_ptx::pack_bf16x2(x - __uint_as_float(p[1] << 16), y - __uint_as_float(p[1] & 0xFFFF0000u));
 }
 
 // Four consecutive fp32 values of row r, columns [c, c + 4), into the three
@@ -85,23 +89,14 @@ __device__ __forceinline__ void split_bf16x3(float x, __nv_bfloat16& p1, __nv_bf
 template <uint32_t PART>
 __device__ __forceinline__ void put_split4(uint8_t* base, int r, int c, float4 v)
 {
-    __nv_bfloat16 p[3][4];
-    split_bf16x3(v.x, p[0][0], p[1][0], p[2][0]);
-    split_bf16x3(v.y, p[0][1], p[1][1], p[2][1]);
-    split_bf16x3(v.z, p[0][2], p[1][2], p[2][2]);
-    split_bf16x3(v.w, p[0][3], p[1][3], p[2][3]);
+    uint32_t lo[3], hi[3];
+    split_pair(v.x, v.y, lo);
+    split_pair(v.z, v.w, hi);
     const int hf = c >> 6, cc = c & 63;  // half, column in the half
     const uint32_t off = hf * (PART / 2) + (r >> 3) * 1024 + (r & 7) * 128 + ((((cc >> 3) ^ (r & 7))) << 4) +
                          (cc & 7) * 2;
 #pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        uint2 w;
-        w.x = static_cast<uint32_t>(__bfloat16_as_ushort(p[s][0])) |
-              (static_cast<uint32_t>(__bfloat16_as_ushort(p[s][1])) << 16);
-        w.y = static_cast<uint32_t>(__bfloat16_as_ushort(p[s][2])) |
-              (static_cast<uint32_t>(__bfloat16_as_ushort(p[s][3])) << 16);
-        *reinterpret_cast<uint2*>(base + s * PART + off) = w;
-    }
+    for (int s = 0; s < 3; ++s) *reinterpret_cast<uint2*>(base + s * PART + off) = make_uint2(lo[s], hi[s]);
 }
 
 struct LtBars {
@@ -150,23 +145,49 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
         s_hi[i] = static_cast<int>(hi);
         s_anchor[i] = anc;
     }
+    __syncthreads();
+    int first = 0;  // first unit with a candidate here (the last one has)
+    for (int last = n_u - 1; first < last;) {
+        const int mid = (first + last) >> 1;
+        if (s_hi[mid] <= b0) first = mid + 1;
+        else last = mid;
+    }
+    const int i0 = first / U, n_it = (n_u + U - 1) / U - i0;
+
     uint8_t* smem = smem_raw + ((1024u - (smem_addr(smem_raw) & 1023u)) & 1023u);
     uint8_t* bbuf = smem;                 // representatives, three parts
     uint8_t* abuf = smem + 3 * kLtBPart;  // two buffers of three parts
+    // the staging warps' rows of tile i; those of the first tile are on their way
+    // while the representatives are staged
+    constexpr int kPer = kLtRows * 32 / kLtStageThreads;
+    const int t = tid - (kLtThreads - kLtStageThreads);
+    float4 v[kPer];
+    auto load_tile = [&](int tile) {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            const int x = t + i * kLtStageThreads, r = x >> 5, c = (x & 31) * 4;
+            const int ul = r / a.g, u = tile * U + ul;
+            v[i] = ul < U && u < n_u
+                       ? __ldg(reinterpret_cast<const float4*>(fp + static_cast<int64_t>(s_anchor[u]) * D +
+                                                               (j * a.g + r - ul * a.g) * kHeadDim + c))
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    };
+    if (t >= 0) load_tile(i0);
     // a warp reads one 512-byte row; eight rows per thread in flight
     for (int x0 = tid; x0 < 128 * 32; x0 += 8 * kLtThreads) {
-        float4 v[8];
+        float4 vb[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int x = x0 + i * kLtThreads, r = x >> 5, c = (x & 31) * 4;
-            v[i] = x < 128 * 32 && b0 + r < a.nb
-                       ? __ldg(reinterpret_cast<const float4*>(reps + (j * a.nb + b0 + r) * kHeadDim + c))
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
+            vb[i] = x < 128 * 32 && b0 + r < a.nb
+                        ? __ldg(reinterpret_cast<const float4*>(reps + (j * a.nb + b0 + r) * kHeadDim + c))
+                        : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int x = x0 + i * kLtThreads;
-            if (x < 128 * 32) put_split4<kLtBPart>(bbuf, x >> 5, (x & 31) * 4, v[i]);
+            if (x < 128 * 32) put_split4<kLtBPart>(bbuf, x >> 5, (x & 31) * 4, vb[i]);
         }
     }
     fence_proxy_async_smem();
@@ -176,7 +197,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
             mbar_init(&bars.a_full[i], kLtStageThreads);
             mbar_init(&bars.a_empty[i], 1);
             mbar_init(&bars.d_full[i], 1);
-            mbar_init(&bars.d_empty[i], 128);
+            mbar_init(&bars.d_empty[i], kLtStoreThreads);
         }
         mbar_init(&bars.drain, 1);
         fence_barrier_init();
@@ -189,14 +210,6 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    int first = 0;  // first unit with a candidate here (the last one has)
-    for (int last = n_u - 1; first < last;) {
-        const int mid = (first + last) >> 1;
-        if (s_hi[mid] <= b0) first = mid + 1;
-        else last = mid;
-    }
-    const int i0 = first / U, n_it = (n_u + U - 1) / U - i0;
-
     if (warp == 0) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
@@ -226,12 +239,14 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
                 mbar_wait_bounded(&bars.drain, 0, a.timeout_ns, nullptr);
             }
         }
-    } else if (warp < 5) {
+    } else if (warp <= kLtStoreThreads / 32) {
         // ------------------------------------------------------------ stores
         const int q = warp & 3;  // TMEM lane quarter this warp may access
-        const uint32_t lane_base = tmem + (static_cast<uint32_t>(q * 32) << 16);
+        const int r0 = warp > 4 ? kLtWarpRows : 0;  // its rows of the tile
+        const uint32_t lane_base = tmem + (static_cast<uint32_t>(q * 32) << 16) + r0;
         const int64_t b = b0 + q * 32 + lane;  // this thread's block
         const bool in = b >= a.n_sink / a.B;
+        const int ul0 = r0 / a.g, left0 = a.g - (r0 - ul0 * a.g);
         for (int it = 0; it < n_it; ++it) {
             const int st = it & 1;
             if (!__all_sync(0xFFFFFFFFu, mbar_wait_bounded(&bars.d_full[st], (it >> 1) & 1, a.timeout_ns, &abort_flag))) {
@@ -239,17 +254,16 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
                 break;
             }
             tc_fence_after();
-            uint32_t z[kLtRows];
-            tmem_ld32(lane_base + st * kLtRows, *reinterpret_cast<uint32_t(*)[32]>(&z[0]));
-            tmem_ld32(lane_base + st * kLtRows + 32, *reinterpret_cast<uint32_t(*)[32]>(&z[32]));
+            uint32_t z[kLtWarpRows];
+            tmem_ld32(lane_base + st * kLtRows, z);
             tmem_ld_wait();
             tc_fence_before();
             mbar_arrive(&bars.d_empty[st]);
-            int ul = (i0 + it) * U, left = a.g;
-            float* dst = logits + (static_cast<int64_t>(u0 + ul) * a.Hq + j * a.g) * a.nb + b;
-            bool live = in && ul < n_u && b < s_hi[ul];
+            int ul = (i0 + it) * U + ul0, left = left0;
+            float* dst = logits + (static_cast<int64_t>(u0 + ul) * a.Hq + j * a.g + a.g - left) * a.nb + b;
+            bool live = in && ul < n_u && ul < (i0 + it + 1) * U && b < s_hi[ul];
 #pragma unroll
-            for (int c = 0; c < kLtRows; ++c) {
+            for (int c = 0; c < kLtWarpRows; ++c) {
                 if (live) *dst = a.sigma * __uint_as_float(z[c]);
                 dst += a.nb;
                 if (--left == 0) {  // the next unit's heads
@@ -262,20 +276,8 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
         }
     } else {
         // ------------------------------------------------------------ staging
-        const int t = tid - 160;
         for (int it = 0; it < n_it; ++it) {
             const int st = it & 1;
-            constexpr int kPer = kLtRows * 32 / kLtStageThreads;
-            float4 v[kPer];
-#pragma unroll
-            for (int i = 0; i < kPer; ++i) {
-                const int x = t + i * kLtStageThreads, r = x >> 5, c = (x & 31) * 4;
-                const int ul = r / a.g, u = (i0 + it) * U + ul;
-                v[i] = ul < U && u < n_u
-                           ? __ldg(reinterpret_cast<const float4*>(fp + static_cast<int64_t>(s_anchor[u]) * D +
-                                                                   (j * a.g + r - ul * a.g) * kHeadDim + c))
-                           : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
             if (it >= 2 && !mbar_wait_bounded(&bars.a_empty[st], ((it >> 1) - 1) & 1, a.timeout_ns, &abort_flag)) {
                 lt_fail(&abort_flag, a.status);
                 break;
@@ -287,6 +289,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
             }
             fence_proxy_async_smem();
             mbar_arrive(&bars.a_full[st]);
+            if (it + 1 < n_it) load_tile(i0 + it + 1);
         }
     }
     tc_fence_before();
