@@ -54,9 +54,11 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 
 constexpr int kDecSlots = 128;     // partial slots per head the workspace is sized for
 constexpr int kDecMaxSplits = 64;  // of which the attention kernel uses at most these
-constexpr int kDecThreads = 256;
-constexpr int kDecWarps = kDecThreads / 32;
-constexpr int kDecStep = 2 * kDecWarps;  // half-warps of a CTA
+// Threads of an attention CTA: one CTA of 512 per SM where a thread's 128
+// registers hold its G query heads, else 256. Half as many CTAs of twice the
+// size leave half the partials for the CTA that merges them.
+template <int G>
+constexpr int dec_threads = G <= 4 ? 512 : 256;
 
 struct DecArgs {
     int Hq, Hkv;
@@ -97,11 +99,14 @@ __host__ __device__ __forceinline__ int64_t window_start(int n_local, int64_t t)
 // Also stores what the step's reuse decision changes: the state words and, when
 // the step retrieved, the anchor.
 template <int G>
-__global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const DecArgs a, const __nv_bfloat16* __restrict__ q,
+__global__ void __launch_bounds__(dec_threads<G>, 1) k_dec_attn(const DecArgs a, const __nv_bfloat16* __restrict__ q,
                                                           const uint4* __restrict__ k,
                                                           const uint4* __restrict__ v,
                                                           __nv_bfloat16* __restrict__ out)
 {
+    constexpr int kDecThreads = dec_threads<G>;
+    constexpr int kDecWarps = kDecThreads / 32;
+    constexpr int kDecStep = 2 * kDecWarps;  // half-warps of the CTA
     constexpr int KB = G <= 2 ? 8 : G <= 4 ? 4 : 2;  // keys per half-warp and update: G KB <= 16
     __shared__ float s_o[kDecWarps][G][kHeadDim];
     __shared__ float2 s_ml[kDecWarps][G];
@@ -158,7 +163,7 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const 
     float m = -INFINITY, l = 0.f;
     const int u_l = c % KB;
     const uint4 zero = make_uint4(0, 0, 0, 0);
-    // half-warp x of the CTA takes the keys i0 + x, i0 + x + 16, ...; lane c
+    // half-warp x of the CTA takes the keys i0 + x, i0 + x + kDecStep, ...; lane c
     // looks up the token of the half-warp's key c of every 16
     for (int b0 = i0 + 2 * warp; b0 < i1; b0 += 16 * kDecStep) {  // warp-uniform
         const int ic = b0 + half + kDecStep * c;
@@ -249,27 +254,22 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const 
         if (lane == 0) s_ml[warp][hl] = make_float2(mm, l1 * w1 + l2 * w2);
     }
     __syncthreads();
-    for (int x = tid; x < G * 32; x += kDecThreads) {
-        const int hl = x >> 5, d4 = x & 31;
+    for (int x = tid; x < G * kHeadDim; x += kDecThreads) {
+        const int hl = x / kHeadDim, dd = x % kHeadDim;
         float mm = -INFINITY;
 #pragma unroll
         for (int w = 0; w < kDecWarps; ++w) mm = fmaxf(mm, s_ml[w][hl].x);
         const float base = mm == -INFINITY ? 0.f : mm;
-        float ll = 0.f;
-        float4 oo = make_float4(0.f, 0.f, 0.f, 0.f);
+        float ll = 0.f, oo = 0.f;
 #pragma unroll
         for (int w = 0; w < kDecWarps; ++w) {
             const float f = ex2(s_ml[w][hl].x - base);
-            const float4 ow = *reinterpret_cast<const float4*>(&s_o[w][hl][4 * d4]);
             ll += s_ml[w][hl].y * f;
-            oo.x += ow.x * f;
-            oo.y += ow.y * f;
-            oo.z += ow.z * f;
-            oo.w += ow.w * f;
+            oo += s_o[w][hl][dd] * f;
         }
         const int64_t slot = static_cast<int64_t>(j * G + hl) * kDecMaxSplits + split;
-        __stcg(&a.o_part[slot * 32 + d4], oo);
-        if (d4 == 0) __stcg(&a.ml_part[slot], make_float2(mm, ll));
+        __stcg(reinterpret_cast<float*>(a.o_part + slot * 32) + dd, oo);
+        if (dd == 0) __stcg(&a.ml_part[slot], make_float2(mm, ll));
     }
     __threadfence();
     __syncthreads();
@@ -298,7 +298,7 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const 
         for (int e = 0; e < kDecMaxSplits / 32; ++e) s_w[hl][lane + 32 * e] = ex2(x[e].x - base) * inv;
     }
     __syncthreads();
-    // warp w sums the splits w, w + 8, ... of every head; s_o takes the warps' sums
+    // warp w sums the splits w, w + kDecWarps, ... of every head; s_o takes the warps' sums
     float4 acc[G];
 #pragma unroll
     for (int hl = 0; hl < G; ++hl) acc[hl] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kDecThreads, G <= 4 ? 2 : 1) k_dec_attn(const 
 template <int G>
 cudaError_t run_dec_attn(const DecArgs& a, const void* q, const void* k, const void* v, void* out, cudaStream_t st)
 {
-    return launch_after(st, dim3(a.Hkv, a.splits), kDecThreads, 0, 1, k_dec_attn<G>, a,
+    return launch_after(st, dim3(a.Hkv, a.splits), dec_threads<G>, 0, 1, k_dec_attn<G>, a,
                         static_cast<const __nv_bfloat16*>(q), static_cast<const uint4*>(k),
                         static_cast<const uint4*>(v), static_cast<__nv_bfloat16*>(out));
 }
@@ -475,11 +475,11 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     }
     if (e != cudaSuccess) return e;
 
-    // Splits: about two CTAs per SM, and at least 64 keys (four per half-warp) each.
+    // Splits: one CTA per SM, and at least 64 keys each.
     int sms = 0;
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int64_t n_max = d.n_sink + static_cast<int64_t>(d.k) + (t - W + 1);
-    int64_t splits = 2 * sms / d.Hkv;
+    int64_t splits = sms / d.Hkv;
     if (splits > (n_max + 63) / 64) splits = (n_max + 63) / 64;
     if (splits > kDecMaxSplits) splits = kDecMaxSplits;
     a.splits = static_cast<int>(splits > 0 ? splits : 1);

@@ -82,17 +82,29 @@ __device__ bool decode_retrieves(const KeyScoreArgs& a)
     const uint4* q = reinterpret_cast<const uint4*>(a.q);
     const float4* an = reinterpret_cast<const float4*>(a.anchor);
     float dot = 0.f, nq = 0.f, na = 0.f;
-    for (int i = threadIdx.x; i < D8; i += kLgThreads) {
-        const uint4 x = q[i];
-        const float4 y0 = an[2 * i], y1 = an[2 * i + 1];
-        const uint32_t w[4] = {x.x, x.y, x.z, x.w};
-        const float y[8] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z, y1.w};
+    constexpr int kIn = 3;  // 32 heads: every load of the thread in flight
+    for (int i0 = threadIdx.x; i0 < D8; i0 += kIn * kLgThreads) {
+        uint4 x[kIn];
+        float4 y0[kIn], y1[kIn];
 #pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            const float v = __uint_as_float(c & 1 ? w[c / 2] & 0xFFFF0000u : w[c / 2] << 16);
-            dot += v * y[c];
-            nq += v * v;
-            na += y[c] * y[c];
+        for (int b = 0; b < kIn; ++b) {
+            const int i = i0 + b * kLgThreads < D8 ? i0 + b * kLgThreads : i0;
+            x[b] = q[i];
+            y0[b] = an[2 * i];
+            y1[b] = an[2 * i + 1];
+        }
+#pragma unroll
+        for (int b = 0; b < kIn; ++b) {
+            if (i0 + b * kLgThreads >= D8) continue;
+            const uint32_t w[4] = {x[b].x, x[b].y, x[b].z, x[b].w};
+            const float y[8] = {y0[b].x, y0[b].y, y0[b].z, y0[b].w, y1[b].x, y1[b].y, y1[b].z, y1[b].w};
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const float v = __uint_as_float(c & 1 ? w[c / 2] & 0xFFFF0000u : w[c / 2] << 16);
+                dot += v * y[c];
+                nq += v * v;
+                na += y[c] * y[c];
+            }
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
