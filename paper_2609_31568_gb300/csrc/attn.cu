@@ -76,6 +76,8 @@ struct AttnArgs {
     int qb_per_sc;     // 128-row query blocks per sub-chunk
     int sc_per_chunk;  // sub-chunks per outer chunk
     int Hq, Hkv, g;
+    int heads;         // query heads (tiles) of a CTA, and
+    int items;         // CTAs per query block and KV head
     int odd_blk;       // query blocks per CTA of an odd group's last head, and
     int odd_per_sc;    // CTAs per sub-chunk and KV head of that head (0: even group)
     int64_t N, nb;
@@ -243,8 +245,8 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
     // comes first, which issues the heaviest rows (longest window) first. ----
     // A work item has two query tiles: two heads of one query block, or, for
     // the last head of an odd group, odd_blk neighbouring query blocks of a
-    // sub-chunk. ----
-    const int per_sc_ctas = a.qb_per_sc * (a.g / 2) + a.odd_per_sc;  // of one KV head
+    // sub-chunk; or one (heads = 1) in a small call. ----
+    const int per_sc_ctas = a.qb_per_sc * a.items + a.odd_per_sc;  // of one KV head
     const int per_chunk_ctas = a.sc_per_chunk * per_sc_ctas * a.Hkv;
     const int c = static_cast<int>(blockIdx.x) / per_chunk_ctas;
     const int sc0 = a.sc_begin + c * a.sc_per_chunk;
@@ -254,17 +256,17 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
     const int kvh = rem / (n_sc * per_sc_ctas);
     rem -= kvh * n_sc * per_sc_ctas;
     if (kvh >= a.Hkv) return;
-    const bool rows2 = rem >= n_qb * (a.g / 2);  // query blocks of one head
+    const bool rows2 = rem >= n_qb * a.items;  // query blocks of one head
     int sc, blk, h0;
     if (!rows2) {
-        const int qb = rem / (a.g / 2);
-        h0 = kvh * a.g + 2 * (rem - qb * (a.g / 2));
+        const int qb = rem / a.items;
+        h0 = kvh * a.g + a.heads * (rem - qb * a.items);
         const int idx = n_qb - 1 - qb;
         sc = idx / a.qb_per_sc;
         blk = idx - sc * a.qb_per_sc;
     } else {
         h0 = kvh * a.g + a.g - 1;
-        const int idx = n_sc * a.odd_per_sc - 1 - (rem - n_qb * (a.g / 2));
+        const int idx = n_sc * a.odd_per_sc - 1 - (rem - n_qb * a.items);
         sc = idx / a.odd_per_sc;
         blk = a.odd_blk * (idx - sc * a.odd_per_sc);
     }
@@ -277,7 +279,7 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
     const int64_t sc_hi = (sc_lo + a.ut.L < e_u) ? sc_lo + a.ut.L : e_u;
     const int64_t q0 = sc_lo + static_cast<int64_t>(kRows) * blk;
     if (q0 >= sc_hi) return;
-    const int nq = !rows2 || (a.odd_blk == 2 && q0 + kRows < sc_hi) ? 2 : 1;  // query tiles of this CTA
+    const int nq = !rows2 ? a.heads : a.odd_blk == 2 && q0 + kRows < sc_hi ? 2 : 1;  // query tiles of this CTA
     const int64_t q_last = rows2 ? q0 + kRows * nq : q0 + kRows;
     const int64_t q_end = q_last < sc_hi ? q_last : sc_hi;
     const int64_t W = (s_u - a.n_local > 0) ? s_u - a.n_local : 0;
@@ -844,17 +846,21 @@ cudaError_t launch_sparse_prefill(const Derived& d, int mode, int64_t tok_begin,
     a.Hq = d.Hq;
     a.Hkv = d.Hkv;
     a.g = d.g;
-    // An odd group's last head: two query blocks per CTA once one block per CTA
-    // would not fit the SMs at a time. A CTA with one query tile runs at the
-    // pace of one softmax chain (8,128 rows of 28 heads on 4, a quarter of the
-    // CTAs with one tile: 691 us; all with two: 627 us), but where
-    // SMs are free twice the CTAs are quicker.
+    // Two heads per CTA share its K and V tiles and overlap one head's softmax
+    // with the other's products. Where every head's tile gets an SM of its own
+    // they run alone: a tile's chain is then not behind another's MMAs (a 4K
+    // layer of 4 heads, 64 CTAs: 39.0 us for its three calls, 128: 38.1 us). An odd group's
+    // last head has two query blocks per CTA once one block per CTA would not
+    // fit the SMs at a time (8,128 rows of 28 heads on 4, a quarter of the CTAs
+    // with one tile: 691 us; all with two: 627 us).
     int sms = 0;
     cudaError_t e = device_sms(&sms);
     if (e != cudaSuccess) return e;
-    const int64_t singles = static_cast<int64_t>(a.n_sc) * d.Hkv * a.qb_per_sc * ((d.g + 1) / 2);
-    a.odd_blk = singles > sms ? 2 : 1;
-    a.odd_per_sc = d.g % 2 ? (a.qb_per_sc + a.odd_blk - 1) / a.odd_blk : 0;
+    const int64_t tiles = static_cast<int64_t>(a.n_sc) * d.Hkv * a.qb_per_sc;  // of one head per KV head
+    a.heads = tiles * d.g <= sms ? 1 : 2;
+    a.items = d.g / a.heads;
+    a.odd_blk = tiles * ((d.g + 1) / 2) > sms ? 2 : 1;
+    a.odd_per_sc = a.heads == 2 && d.g % 2 ? (a.qb_per_sc + a.odd_blk - 1) / a.odd_blk : 0;
     a.N = d.N;
     a.nb = d.nb;
     a.B = d.B;
@@ -886,7 +892,7 @@ cudaError_t launch_sparse_prefill(const Derived& d, int mode, int64_t tok_begin,
     auto kern = tok ? k_sparse_attn<true> : k_sparse_attn<false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemBytes));
     if (e != cudaSuccess) return e;
-    const int64_t grid = static_cast<int64_t>(a.n_sc) * d.Hkv * (a.qb_per_sc * (d.g / 2) + a.odd_per_sc);
+    const int64_t grid = static_cast<int64_t>(a.n_sc) * d.Hkv * (a.qb_per_sc * a.items + a.odd_per_sc);
     if (grid <= 0 || grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
     return launch_after(st, dim3(static_cast<unsigned>(grid)), kThreads, kSmemBytes, 1, kern, tq, tk, tv, tpk, tpv, a);
 }
