@@ -395,6 +395,8 @@ constexpr int kTopkThreads = 1024;
 constexpr int kSortMax = 4096;     // candidates up to which k_topk and k_select_fused keep the keys in shared memory
 
 constexpr int kRadixBins = 2048;   // digits of 11, 11 and 10 bits
+constexpr int kTopkPad = 128;
+constexpr int kTopkCount = 256;    // keys up to which topk_emit counts instead
 
 // Shared memory of topk_emit.
 struct TopkShared {
@@ -408,14 +410,53 @@ struct TopkShared {
 // largest key T (three passes over the keys, each a histogram and one block
 // scan of its bins), then the keys above T and the first ones equal to it, in
 // index order (every warp owns a run of keys: counts, one scan, ballots).
-// About 4 us for 1024 keys; the 55 exchange steps of a bitonic sort of 64-bit
-// keys took 8. Called by all THREADS threads of the CTA.
+// About 3 us for 1024 keys (the 55 exchange steps of a bitonic sort of 64-bit
+// keys took 8). `keys` is 16-byte aligned, with room for kTopkPad more. Called
+// by all THREADS threads of the CTA.
 template <int THREADS>
-__device__ void topk_emit(const uint32_t* keys, int n, int64_t lo, int k, int32_t* out, TopkShared& sh)
+__device__ void topk_emit(uint32_t* keys, int n, int64_t lo, int k, int32_t* out, TopkShared& sh)
 {
     constexpr int kWarps = THREADS / 32;
     constexpr int kPer = kRadixBins / THREADS;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (n <= kTopkCount) {
+        // Few keys: `per` threads per key count the keys ahead of it (larger, or
+        // equal with a lower index); fewer than k make it a pick. The work grows
+        // with n^2: against the three passes it saves 1.2 us per call at 250 keys,
+        // 2 us at 60, and nothing at 500.
+        int per = THREADS / kTopkCount;
+        while (per < 32 && 2 * per * n <= THREADS) per *= 2;
+        const int n_pad = (n + 4 * per - 1) / (4 * per) * (4 * per);
+        if (tid < n_pad - n) keys[n + tid] = 0u;  // ahead of no key
+        __syncthreads();
+        const int i = tid / per, part = tid % per;
+        const uint32_t mine = i < n ? keys[i] : 0u;
+        int above = 0, level = 0;
+#pragma unroll 4
+        for (int x = 4 * part; x < n_pad; x += 4 * per) {
+            const uint4 v = *reinterpret_cast<const uint4*>(keys + x);
+            above += (v.x > mine) + (v.y > mine) + (v.z > mine) + (v.w > mine);
+            level += (v.x >= mine) + (v.y >= mine) + (v.z >= mine) + (v.w >= mine);
+        }
+        for (int o = per / 2; o > 0; o >>= 1) {
+            above += __shfl_xor_sync(0xFFFFFFFFu, above, o);
+            level += __shfl_xor_sync(0xFFFFFFFFu, level, o);
+        }
+        if (__any_sync(0xFFFFFFFFu, i < n && level > above + 1)) {  // ties: the lower index first
+            int ties = 0;
+            for (int x = part; x < i && x < n; x += per) ties += keys[x] == mine;
+            for (int o = per / 2; o > 0; o >>= 1) ties += __shfl_xor_sync(0xFFFFFFFFu, ties, o);
+            above += ties;
+        }
+        const bool pick = i < n && above < k && part == 0;
+        const unsigned b = __ballot_sync(0xFFFFFFFFu, pick);
+        if (lane == 0) sh.scan[warp] = __popc(b);
+        __syncthreads();
+        int before = lane < warp ? sh.scan[lane] : 0;
+        for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xFFFFFFFFu, before, o);
+        if (pick) out[before + __popc(b & ((1u << lane) - 1u))] = static_cast<int32_t>(lo + i);
+        return;
+    }
     uint32_t prefix = 0;
     int need = k;
     for (int p = 0; p < 3; ++p) {
@@ -513,7 +554,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
 {
     __shared__ int hist[256];
     __shared__ __align__(16) int whist[kTopkThreads / 32][256];  // per-warp histograms, or keys and scratch
-    static_assert(sizeof(whist) >= kSortMax * sizeof(uint32_t) + sizeof(TopkShared), "key buffer");
+    static_assert(sizeof(whist) >= (kSortMax + kTopkPad) * sizeof(uint32_t) + sizeof(TopkShared), "key buffer");
     __shared__ uint32_t s_prefix;
     __shared__ int s_need;
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
@@ -542,7 +583,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
         uint32_t* sk = reinterpret_cast<uint32_t*>(&whist[0][0]);
         for (int i = threadIdx.x; i < n; i += blockDim.x) sk[i] = float_key(sc[lo + i]);
         __syncthreads();
-        topk_emit<kTopkThreads>(sk, static_cast<int>(n), lo, a.k, out, *reinterpret_cast<TopkShared*>(sk + kSortMax));
+        topk_emit<kTopkThreads>(sk, static_cast<int>(n), lo, a.k, out, *reinterpret_cast<TopkShared*>(sk + kSortMax + kTopkPad));
         if (threadIdx.x == 0) sel_count[u] = a.k;  // n > k: exactly k picks
         return;
     }
@@ -700,7 +741,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
                                                                int32_t* __restrict__ sel_count)
 {
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
-    __shared__ uint32_t sk[kSortMax];
+    __shared__ __align__(16) uint32_t sk[kSortMax + kTopkPad];
     __shared__ TopkShared sh;
     scale_ptx::pdl_enter();
     const int u_first = unit_lower_bound(a.ut, a.sc_begin);
@@ -849,7 +890,7 @@ __device__ __forceinline__ void reduce_to_lanes(float (&v)[V])
 // the GPU); 32 calls of a 32K layer take 0.43 ms less. Beyond kFewUnits the
 // 16-fold reads of the representatives and the rounds of clusters cost more
 // than the two kernels (64 units: eight rounds against 69 us).
-// Dynamic shared memory: logits [H_q][stride], then keys [nb].
+// Dynamic shared memory: logits [H_q][stride], then keys [nb + kTopkPad].
 template <int G>
 __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const float* __restrict__ fp,
                                                                const float* __restrict__ reps, int stride,
@@ -918,14 +959,29 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     }
     cluster_wait();
     __syncthreads();
-    // (max, sum) of the run per head, to every rank: lane x sends to rank x % 16
-    for (int h = warp; h < a.Hq; h += kFewWarps) {
-        float m = -INFINITY, sum = 0.f;
-        for (int i = lane; i < len; i += 32) m = fmaxf(m, zs[h * stride + i]);
-        for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-        for (int i = lane; i < len; i += 32) sum += expf(zs[h * stride + i] - m);
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        if (lane < kFewCtas) st_cluster_f2(cluster_map(&s_part[rank][h], lane), m, sum);
+    // (max, sum) of the run per head, to every rank (lane r to rank r); two heads
+    // of a warp at a time, their chains side by side
+    for (int h0 = warp; h0 < a.Hq; h0 += 2 * kFewWarps) {
+        float m[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};
+        const float* zh[2] = {zs + h0 * stride, zs + (h0 + kFewWarps < a.Hq ? h0 + kFewWarps : h0) * stride};
+        for (int i = lane; i < len; i += 32)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) m[c] = fmaxf(m[c], zh[c][i]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) m[c] = fmaxf(m[c], __shfl_xor_sync(0xFFFFFFFFu, m[c], o));
+        for (int i = lane; i < len; i += 32)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) sum[c] += expf(zh[c][i] - m[c]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) sum[c] += __shfl_xor_sync(0xFFFFFFFFu, sum[c], o);
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+            if (lane < kFewCtas && h0 + c * kFewWarps < a.Hq)
+                st_cluster_f2(cluster_map(&s_part[rank][h0 + c * kFewWarps], lane), m[c], sum[c]);
     }
     cluster_arrive();
     cluster_wait();
@@ -966,7 +1022,7 @@ FewPlan few_plan(const Derived& d, int max_units)
     FewPlan p{0, 0};
     if (max_units > kFewUnits || d.g > 8 || d.Hq > kFusedMaxHeads) return p;
     const int64_t stride = ((d.nb + kFewCtas - 1) / kFewCtas + 7) / 8 * 8;
-    const int64_t bytes = (stride * d.Hq + d.nb) * 4;
+    const int64_t bytes = (stride * d.Hq + d.nb + kTopkPad) * 4;
     if (bytes > kFewSmem - 48 * 1024) return p;
     p.stride = static_cast<int>(stride);
     p.smem = static_cast<size_t>(bytes);
