@@ -39,6 +39,8 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p)
 constexpr int kFpWarps = 16;
 constexpr int kFpGroupCols = 32;  // sixteen-byte columns of a fingerprint CTA
 constexpr int kStepThreads = 32 * kFpWarps;
+constexpr int kBand = 4096;       // cosines that the clustering keeps in shared memory
+static_assert(kBand * sizeof(float) <= kStepThreads * 2 * sizeof(float4), "k_step_a's buffer");
 
 struct StepArgs {
     const uint4* q;
@@ -219,7 +221,7 @@ __device__ int block_exclusive_scan(int f, int* sh, int* total)
 // chunk walks its sub-chunks: the anchor a admits j while cos(v_a, v_j) >=
 // theta and |C_a| < S_max), which then compacts the anchor flags of those chunks
 // into unit_start, after the *n_units units of the chunks before c_begin.
-__device__ void cluster(const StepArgs& a, int* sh)
+__device__ void cluster(const StepArgs& a, int* sh, float* band)
 {
     const int M = a.M, S_max = a.S_max, per_outer = a.per_outer, c_begin = a.c_begin, c_end = a.c_end;
     const float theta = a.theta;
@@ -231,15 +233,15 @@ __device__ void cluster(const StepArgs& a, int* sh)
     int offset = c_begin == 0 ? 0 : *n_units;
     const int m_begin = c_begin * per_outer;
     const int m_end = min(M, c_end * per_outer);
-    for (int c = c_begin + static_cast<int>(threadIdx.x); c < c_end; c += blockDim.x) {
-        const int c0 = c * per_outer;
-        const int c1 = min(M, c0 + per_outer);
-        int an = c0;
+    // cosine of sub-chunk an with sub-chunk j: cs(an, j - an)
+    auto walk = [&](int c, auto cs) {
+        const int c1 = min(M, (c + 1) * per_outer);
+        int an = c * per_outer;
         while (an < c1) {
             flag[an] = 1;
             int size = 1, j = an + 1;
             while (j < c1 && size < S_max) {
-                const bool admit = always || __ldcg(&a.gram[static_cast<int64_t>(an) * S_max + (j - an)]) >= theta;
+                const bool admit = always || cs(an, j - an) >= theta;
                 if (!admit) break;
                 flag[j] = 0;
                 ++size;
@@ -247,6 +249,27 @@ __device__ void cluster(const StepArgs& a, int* sh)
             }
             an = j;
         }
+    };
+    // The walk is a chain of dependent cosines: their band is brought into shared
+    // memory, as many chunks at a time as fit (16 chunks of 16 sub-chunks: 30
+    // cycles a link instead of 700).
+    const int64_t per_chunk = static_cast<int64_t>(per_outer) * S_max;
+    if (!always && per_chunk <= kBand) {
+        const int batch = min(static_cast<int>(kBand / per_chunk), static_cast<int>(blockDim.x));
+        for (int cb = c_begin; cb < c_end; cb += batch) {
+            const int row0 = cb * per_outer;
+            const int rows = min(m_end, (cb + batch) * per_outer) - row0;
+            for (int i = threadIdx.x; i < rows * S_max; i += blockDim.x)
+                band[i] = __ldcg(&a.gram[static_cast<int64_t>(row0) * S_max + i]);
+            __syncthreads();
+            const int c = cb + static_cast<int>(threadIdx.x);
+            if (static_cast<int>(threadIdx.x) < batch && c < c_end)
+                walk(c, [&](int an, int d) { return band[(an - row0) * S_max + d]; });
+            __syncthreads();
+        }
+    } else {
+        for (int c = c_begin + static_cast<int>(threadIdx.x); c < c_end; c += blockDim.x)
+            walk(c, [&](int an, int d) { return __ldcg(&a.gram[static_cast<int64_t>(an) * S_max + d]); });
     }
     __syncthreads();
     for (int base = m_begin; base < m_end; base += blockDim.x) {
@@ -269,6 +292,7 @@ __global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __rest
 {
     __shared__ int sh[40];
     __shared__ int last;
+    __shared__ float band[kBand];
     scale_ptx::pdl_enter();
     const float* fp = args.fp;
     const float* ss_part = args.ss_part;
@@ -303,14 +327,14 @@ __global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __rest
     __syncthreads();
     if (!last) return;
     __threadfence();
-    cluster(args, sh);
+    cluster(args, sh, band);
 }
 
 // Roles by CTA: the clusters where they need no cosine (one CTA), then the
 // fingerprints, then the representatives, whose CTAs fill the SMs that the
 // fingerprints of a short range leave free. Bound by HBM: 128K tokens of 32
-// query and 8 KV heads (1.35 GB) with a threshold take 206 us with k_gram,
-// 6.6 TB/s (222 us as four kernels); chunk by chunk with theta = -1 the eight
+// query and 8 KV heads (1.35 GB) with a threshold take 199 us with k_gram,
+// 6.8 TB/s (222 us as four kernels); chunk by chunk with theta = -1 the eight
 // calls of that layer take 0.25 ms less, a 4K layer's one call 14 us less.
 __global__ void __launch_bounds__(kStepThreads, 2) k_step_a(const StepArgs a)
 {
@@ -321,7 +345,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_step_a(const StepArgs a)
     int x = blockIdx.x;
     if (x == 0) {
         if (threadIdx.x == 0) *a.ticket = 0;
-        if (a.theta <= -1.0f || a.S_max == 1) cluster(a, sh);
+        if (a.theta <= -1.0f || a.S_max == 1) cluster(a, sh, reinterpret_cast<float*>(part));
         return;
     }
     --x;
