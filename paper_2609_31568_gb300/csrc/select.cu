@@ -41,7 +41,8 @@ __device__ __forceinline__ void cand_range(const SelArgs& a, int64_t s, int64_t*
 {
     const int64_t W = s - a.n_local > 0 ? s - a.n_local : 0;
     *lo = a.n_sink / a.B;                 // first block with (b+1)B > n_sink
-    *hi = (W + a.B - 1) / a.B;            // one past the last block with bB < W
+    // one past the last block with bB < W (both below 2^31: a 32-bit division)
+    *hi = (static_cast<uint32_t>(W) + static_cast<uint32_t>(a.B) - 1u) / static_cast<uint32_t>(a.B);
     if (*hi > a.nb) *hi = a.nb;
     if (*hi < *lo) *hi = *lo;
 }
@@ -1403,6 +1404,7 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
         const cudaError_t ef = launch_select_few(d, a, few, max_units, fingerprints, reps, sel_scores, sel_blocks,
                                                  sel_count, st);
         if (ef == cudaSuccess) return ef;
+        cudaGetLastError();
     }
     // Tiles per CTA: as many as leave every SM a CTA, at most kLtSeg.
     int sms = 0;
