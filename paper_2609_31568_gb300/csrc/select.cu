@@ -11,7 +11,7 @@
 //             compaction (up to 4096 candidates in shared memory; with a
 //             scratch area and more than 64K candidates, the multi-CTA form
 //             below): output ascending, ties to the lower b.
-// Calls of at most 16 units run in one kernel instead, k_select_few.
+// Calls of few units run in one kernel instead, k_select_few.
 //
 // Candidates of unit u are the blocks with a token in [n_sink, W_u),
 // W_u = max(0, s_u - n_local): the contiguous range [b_lo, b_hi(u)).
@@ -856,7 +856,8 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
 constexpr int kFewCtas = 16;       // CTAs of a unit's cluster
 constexpr int kFewThreads = 512;
 constexpr int kFewWarps = kFewThreads / 32;
-constexpr int kFewUnits = 16;      // most units per call (two rounds of the eight or nine clusters that fit at once)
+constexpr int kFewUnits = 16;      // most units per call
+constexpr int kFewClusters = 7;    // clusters of 16 that run at once
 constexpr int kFewSmem = 200 * 1024;
 
 // Values v[0..V) of every lane summed over the 32 lanes: lane c ends with the
@@ -886,11 +887,17 @@ __device__ __forceinline__ void reduce_to_lanes(float (&v)[V])
 // k largest. Nothing but the selection (and the scores, if asked for) is
 // written to memory. Bound by latency: reading 4 MB of representatives at
 // 128K tokens takes the 16 SMs about 2 us, the three exchanges and the top-k
-// the rest. A call for one unit of that layer takes 23 us from Python, most of
-// it the host's, against 35 us with k_logits and k_select_fused (16 + 15 us on
-// the GPU); 32 calls of a 32K layer take 0.43 ms less. Beyond kFewUnits the
-// 16-fold reads of the representatives and the rounds of clusters cost more
-// than the two kernels (64 units: eight rounds against 69 us).
+// the rest. Seven clusters run at once, so a call takes (GPU time, 32 heads)
+//   units               1     8    15   |  k_logits + k_select_fused
+//     64 blocks       5.2   9.5  13.7   |  15
+//    256              8.1  13.0  17.9   |  17
+//    512              9.7  15.5  21.5   |  17.4
+//   1024             12.0  20.6  29     |  18.4
+//   2048             16.7  29.5  42     |  22 us
+// and proportionally less with fewer heads: few_plan takes two rounds up to
+// 2^14 logits per unit, a third up to 2^11. In calls per cluster the host
+// knows only the number of sub-chunks, and the clusters are as a rule a few:
+// those calls stay here up to kFewUnits.
 // Dynamic shared memory: logits [H_q][stride], then keys [nb + kTopkPad].
 template <int G>
 __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const float* __restrict__ fp,
@@ -1018,10 +1025,13 @@ struct FewPlan {
     int stride;
     size_t smem;
 };
-FewPlan few_plan(const Derived& d, int max_units)
+FewPlan few_plan(const Derived& d, bool per_subchunk, int max_units)
 {
     FewPlan p{0, 0};
     if (max_units > kFewUnits || d.g > 8 || d.Hq > kFusedMaxHeads) return p;
+    const int64_t logits = static_cast<int64_t>(d.nb) * d.Hq;
+    const int rounds = logits <= (1 << 11) ? 3 : logits <= (1 << 14) ? 2 : 1;
+    if (per_subchunk && max_units > rounds * kFewClusters) return p;
     const int64_t stride = ((d.nb + kFewCtas - 1) / kFewCtas + 7) / 8 * 8;
     const int64_t bytes = (stride * d.Hq + d.nb + kTopkPad) * 4;
     if (bytes > kFewSmem - 48 * 1024) return p;
@@ -1397,7 +1407,7 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
     const int max_units = a.sc_end - a.sc_begin;  // units in range <= sub-chunks in range
     if (max_units <= 0) return cudaSuccess;
 
-    const FewPlan few = few_plan(d, max_units);
+    const FewPlan few = few_plan(d, a.ut.per_subchunk, max_units);
     if (few.stride) {
         // A cluster of 16 may not be had everywhere (a partition of the device);
         // nothing is enqueued then and the kernels below do the work.

@@ -36,6 +36,10 @@ CASES = [
     (32, 8, 70000, 10000, 16, 64, 128, 1000, 7, True),  # more blocks than the shared memory holds
     (4, 2, 3000, 1000, 64, 64, 128, 0, 3, False),     # nothing selected
     (4, 1, 300000, 10000, 64, 64, 1024, 64, 30, True),  # many units, 4,688 blocks
+    (32, 8, 16416, 1000, 32, 0, 0, 64, 7, True),     # 513 x 32 logits a unit: one round of clusters
+    (32, 8, 16416, 1000, 32, 0, 0, 64, 8, True),     # and one unit more
+    (32, 8, 16384, 1024, 32, 0, 0, 64, 14, False),   # 2^14: two rounds
+    (32, 8, 16384, 1024, 32, 0, 0, 64, 15, False),
 ]
 
 
