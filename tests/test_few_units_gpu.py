@@ -31,6 +31,9 @@ CASES = [
     (16, 16, 3000, 1000, 0, 64, 0, False),    # nothing selected
     (1, 1, 40000, 20000, 128, 512, 19000, True),
     (32, 8, 30011, 2048, 128, 1024, 2000, False),
+    # keys larger than L2 keeps: the unit tiles side by side, the last of two units and of one
+    (32, 8, 50001, 2048, 128, 1024, 2000, False),
+    (28, 4, 100003, 8192, 130, 128, 300, True),
     # slices longer than the keys that stay in shared memory
     (1, 1, 10_400_003, 5_200_064, 128, 0, 30000, False),
 ]
