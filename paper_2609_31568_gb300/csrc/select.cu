@@ -910,11 +910,11 @@ __device__ __forceinline__ void reduce_to_lanes(float (&v)[V])
 // 128K tokens takes the 16 SMs about 2 us, the three exchanges and the top-k
 // the rest. Seven clusters run at once, so a call takes (GPU time, 32 heads)
 //   units               1     8    15   |  k_logits + k_select_fused
-//     64 blocks       5.2   9.5  13.7   |  15
-//    256              8.1  13.0  17.9   |  17
+//     64 blocks       5.8   9.8  14.2   |  15
+//    256              8.0  13.1  18     |  17
 //    512              9.7  15.5  21.5   |  17.4
-//   1024             12.0  20.6  29     |  18.4
-//   2048             16.7  29.5  42     |  22 us
+//   1024             12.1  20.6  29     |  18.4
+//   2048             16.9  29.5  42     |  22 us
 // and proportionally less with fewer heads: few_plan takes two rounds up to
 // 2^14 logits per unit, a third up to 2^11. In calls per cluster the host
 // knows only the number of sub-chunks, and the clusters are as a rule a few:
@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     constexpr int NB = G <= 4 ? 8 : 4;
     constexpr int V = G == 1 ? 8 : G == 2 ? 16 : 32;
     extern __shared__ float zs[];
-    __shared__ float2 s_part[kFewCtas][kFusedMaxHeads];
+    __shared__ float2 s_part[kFewCtas][kFusedMaxHeads + 1];  // + 1: a head's ranks in different banks
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
     __shared__ TopkShared sh;
     pdl_enter();
