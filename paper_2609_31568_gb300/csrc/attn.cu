@@ -166,13 +166,16 @@ __device__ __forceinline__ bool mma_iteration(Barriers* bars, uint32_t tmem, uin
 
 // The MMA issue loop, run by one thread: T iterations (two per trip, so the
 // stage indices are constants), then the last P.V and the O-ready commit.
-// This thread is the critical path: NQ is a compile-time constant and all
-// state is held in registers. Returns false when a wait ran out or the
-// kernel was aborted.
+// `skip_last`: the last key tile lies in the future of every row of query tile
+// 0 (two query blocks of one head), which leaves its P.V out: P is 0, and 0
+// times an infinite value row is NaN. This thread is the critical path: NQ is
+// a compile-time constant and all state is held in registers. Returns false
+// when a wait ran out or the kernel was aborted.
 template <int NQ>
 __device__ __forceinline__ bool mma_issue_loop(Barriers* bars, uint32_t tmem, uint64_t qdesc0, uint64_t kdesc0,
                                                uint64_t vdesc0, uint32_t id_qk, uint32_t id_pv, int T,
-                                               uint64_t timeout_ns, const volatile int* abort_flag)
+                                               bool skip_last, uint64_t timeout_ns,
+                                               const volatile int* abort_flag)
 {
     constexpr uint64_t kStageStep = kTileBytes >> 4;
     int t = 0;
@@ -188,6 +191,7 @@ __device__ __forceinline__ bool mma_issue_loop(Barriers* bars, uint32_t tmem, ui
     for (int qt = 0; qt < NQ; ++qt) {
         if (!mbar_wait_bounded(&bars->p_full[qt], (T - 1) & 1, timeout_ns, abort_flag)) return false;
         tc_fence_after();
+        if (NQ == 2 && qt == 0 && skip_last) continue;
         mma_ts_k128<2048>(tmem + qt * 256 + 128, tmem + qt * 256, vdesc0 + ((T - 1) & 1) * kStageStep, id_pv,
                           T > 1 ? 1u : 0u);
     }
@@ -474,10 +478,11 @@ k_sparse_attn(const __grid_constant__ CUtensorMap tq, const __grid_constant__ CU
             const uint64_t kdesc0 = sdesc_sw128(k_base, 16, 1024);
             const uint64_t vdesc0 = sdesc_sw128(v_base, kHalf, 1024);
             if (ok)
-                ok = nq == 2 ? mma_issue_loop<2>(&bars, tmem, qdesc0, kdesc0, vdesc0, id_qk, id_pv, T, a.timeout_ns,
+                ok = nq == 2 ? mma_issue_loop<2>(&bars, tmem, qdesc0, kdesc0, vdesc0, id_qk, id_pv, T,
+                                                 rows2 && W + 128ll * (n_lt - 1) >= q0 + kRows, a.timeout_ns,
                                                  &abort_flag)
-                             : mma_issue_loop<1>(&bars, tmem, qdesc0, kdesc0, vdesc0, id_qk, id_pv, T, a.timeout_ns,
-                                                 &abort_flag);
+                             : mma_issue_loop<1>(&bars, tmem, qdesc0, kdesc0, vdesc0, id_qk, id_pv, T, false,
+                                                 a.timeout_ns, &abort_flag);
             if (!ok) {
                 fail(&abort_flag, a.status);
                 // Drain: every MMA issued so far completes before TMEM is freed.
