@@ -11,7 +11,7 @@
 //             compaction (up to 4096 candidates in shared memory; with a
 //             scratch area and more than 64K candidates, the multi-CTA form
 //             below): output ascending, ties to the lower b.
-// Calls of few units run in one kernel instead, k_select_few.
+// Sequences of little selection work run in one kernel instead, k_select_few.
 //
 // Candidates of unit u are the blocks with a token in [n_sink, W_u),
 // W_u = max(0, s_u - n_local): the contiguous range [b_lo, b_hi(u)).
@@ -871,16 +871,12 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
     if (threadIdx.x == 0) sel_count[u] = a.k;  // n > k: exactly k picks
 }
 
-// ---- a few units (every call of the Algorithm 2 loop): the whole selection
-// in one launch.
+// ---- sequences of little selection work: the whole selection in one launch.
 
-constexpr int kFewCtas = 16;       // CTAs of a unit's cluster
+constexpr int kFewRuns = 16;       // runs of a unit's candidates, each with a partial softmax sum
 constexpr int kFewThreads = 512;
 constexpr int kFewWarps = kFewThreads / 32;
-constexpr int kFewUnits = 16;      // most units per call
-constexpr int kFewClusters = 7;    // clusters of 16 that run at once
-constexpr int kFewSmem = 200 * 1024;
-
+constexpr int kFewSmem = 152 * 1024;
 // Values v[0..V) of every lane summed over the 32 lanes: lane c ends with the
 // sum of value c % V in v[0] (halving exchanges: V - 1 shuffles, then log2(32 / V)).
 template <int V>
@@ -899,28 +895,24 @@ __device__ __forceinline__ void reduce_to_lanes(float (&v)[V])
     for (int x = V; x < 32; x <<= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], x);
 }
 
-// A cluster of 16 CTAs per unit, rank r owning a run of the unit's candidate
-// blocks. Logits: a warp takes NB blocks of one KV head at a time, each lane
-// four of the 128 dimensions of the representatives and of the head's G
-// queries, in fp32; they stay in shared memory. Statistics: (max, sum) of the
-// run for every head, sent to all ranks. Vote: the ranks' (max, sum) merged in
-// order, then the scores of the run, whose keys go to rank 0, which picks the
-// k largest. Nothing but the selection (and the scores, if asked for) is
-// written to memory. Bound by latency: reading 4 MB of representatives at
-// 128K tokens takes the 16 SMs about 2 us, the three exchanges and the top-k
-// the rest. Seven clusters run at once, so a call takes (GPU time, 32 heads)
-//   units               1     8    15   |  k_logits + k_select_fused
-//     64 blocks       5.8   9.8  14.2   |  15
-//    256              8.0  13.1  18     |  17
-//    512              9.7  15.5  21.5   |  17.4
-//   1024             12.1  20.6  29     |  18.4
-//   2048             16.9  29.5  42     |  22 us
-// and proportionally less with fewer heads: few_plan takes two rounds up to
-// 2^14 logits per unit, a third up to 2^11. In calls per cluster the host
-// knows only the number of sub-chunks, and the clusters are as a rule a few:
-// those calls stay here up to kFewUnits.
-// Dynamic shared memory: logits [H_q][stride], then keys [nb + kTopkPad].
-template <int G>
+// A cluster of gridDim.x (1, 2, .. 16) CTAs per unit. The unit's candidate
+// blocks are cut into 16 runs, of which every rank owns 16 / gridDim.x
+// neighbouring ones. Logits: a warp takes NB blocks of one KV head at a time,
+// each lane four of the 128 dimensions of the representatives and of the head's
+// G queries, in fp32; they stay in shared memory. Statistics: (max, sum) of
+// every run for every head, sent to all ranks. Vote: the runs' (max, sum) merged
+// in order, then the scores of the rank's blocks, whose keys go to rank 0, which
+// picks the k largest. Nothing but the selection (and the scores, if asked for)
+// is written to memory. The arithmetic depends on the unit alone, not on the
+// size of the cluster or on the other units of the call: a unit has the same
+// scores, bit for bit, in every call. Bound by latency in a large cluster, by
+// the shuffles of the dot products and the reads of the representatives from L2
+// in a small one (the next item's blocks in flight during them: 1024 x 32 logits
+// on one CTA 91 us against 83, not taken); few_ctas chooses by the number of units.
+// Dynamic shared memory: logits [H_q][runs of the rank * stride], then keys
+// [nb + kTopkPad]. RUNS: runs of a rank, 0 when gridDim.x decides; as a constant
+// they save 0.3 us of 5.5 in a cluster of 16.
+template <int G, int RUNS>
 __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const float* __restrict__ fp,
                                                                const float* __restrict__ reps, int stride,
                                                                float* __restrict__ scores,
@@ -931,7 +923,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     constexpr int NB = G <= 4 ? 8 : 4;
     constexpr int V = G == 1 ? 8 : G == 2 ? 16 : 32;
     extern __shared__ float zs[];
-    __shared__ float2 s_part[kFewCtas][kFusedMaxHeads + 1];  // + 1: a head's ranks in different banks
+    __shared__ float2 s_part[kFewRuns][kFusedMaxHeads + 1];  // + 1: a head's runs in different banks
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
     __shared__ TopkShared sh;
     pdl_enter();
@@ -943,11 +935,13 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     cand_range(a, s, &lo, &hi);
     const int n = static_cast<int>(hi - lo);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int ctas = RUNS ? kFewRuns / RUNS : static_cast<int>(gridDim.x);
+    const int runs = RUNS ? RUNS : kFewRuns / ctas;  // of this rank
     const int rank = static_cast<int>(cluster_ctarank());
     float* sc = scores ? scores + static_cast<int64_t>(u) * a.nb : nullptr;
     int32_t* out = sel + static_cast<int64_t>(u) * a.k;
     if (sc)  // NaN off the candidates
-        for (int64_t b = rank * kFewThreads + tid; b < a.nb; b += kFewCtas * kFewThreads)
+        for (int64_t b = rank * kFewThreads + tid; b < a.nb; b += ctas * kFewThreads)
             if (b < lo || b >= hi) sc[b] = __int_as_float(0x7FC00000);
     const bool pick = n > a.k && a.k > 0;
     if (!pick) {  // every candidate, or none
@@ -958,12 +952,13 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
         if (!sc || n == 0) return;
     }
     cluster_arrive();  // waited for before the first store to another rank: all have started
-    const int slice = ((n + kFewCtas - 1) / kFewCtas + NB - 1) / NB * NB;  // at most `stride`
-    const int r0 = rank * slice;
-    const int len = n - r0 < slice ? (n - r0 > 0 ? n - r0 : 0) : slice;
+    const int slice = ((n + kFewRuns - 1) / kFewRuns + NB - 1) / NB * NB;  // blocks of a run, at most `stride`
+    const int row = runs * stride;                                         // logits of a head
+    const int r0 = rank * runs * slice;
+    const int len = n - r0 < runs * slice ? (n - r0 > 0 ? n - r0 : 0) : runs * slice;
     const int Hkv = a.Hq / G;
 
-    // logits of the run: items (KV head, NB blocks), a KV head's items on neighbouring warps
+    // logits of the rank's blocks: items (KV head, NB blocks), a KV head's items on neighbouring warps
     const int nbk = (len + NB - 1) / NB;
     for (int it = warp; it < nbk * Hkv; it += kFewWarps) {
         const int j = it / nbk, b0 = (it - j * nbk) * NB;
@@ -984,23 +979,26 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
                 v[hl * NB + i] = fmaf(qv.x, x[i].x, qv.y * x[i].y) + fmaf(qv.z, x[i].z, qv.w * x[i].w);
         }
         reduce_to_lanes<V>(v);
-        if (lane < G * NB) zs[(j * G + lane / NB) * stride + b0 + lane % NB] = a.sigma * v[0];
+        if (lane < G * NB) zs[(j * G + lane / NB) * row + b0 + lane % NB] = a.sigma * v[0];
     }
     cluster_wait();
     __syncthreads();
-    // (max, sum) of the run per head, to every rank (lane r to rank r); two heads
-    // of a warp at a time, their chains side by side
-    for (int h0 = warp; h0 < a.Hq; h0 += 2 * kFewWarps) {
+    // (max, sum) of every run per head, to every rank (lane r to rank r); a warp
+    // takes heads h and h + half of a run at a time, their chains side by side
+    const int half = (a.Hq + 1) / 2;
+    for (int x = warp; x < runs * half; x += kFewWarps) {
+        const int run = runs == 1 ? 0 : x / half, h0 = x - run * half;
+        const int cnt = len - run * slice < slice ? len - run * slice : slice;
         float m[2] = {-INFINITY, -INFINITY}, sum[2] = {0.f, 0.f};
-        const float* zh[2] = {zs + h0 * stride, zs + (h0 + kFewWarps < a.Hq ? h0 + kFewWarps : h0) * stride};
-        for (int i = lane; i < len; i += 32)
+        const float* zh[2] = {zs + h0 * row + run * slice, zs + (h0 + half < a.Hq ? h0 + half : h0) * row + run * slice};
+        for (int i = lane; i < cnt; i += 32)
 #pragma unroll
             for (int c = 0; c < 2; ++c) m[c] = fmaxf(m[c], zh[c][i]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
             for (int c = 0; c < 2; ++c) m[c] = fmaxf(m[c], __shfl_xor_sync(0xFFFFFFFFu, m[c], o));
-        for (int i = lane; i < len; i += 32)
+        for (int i = lane; i < cnt; i += 32)
 #pragma unroll
             for (int c = 0; c < 2; ++c) sum[c] += expf(zh[c][i] - m[c]);
 #pragma unroll
@@ -1009,32 +1007,32 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
             for (int c = 0; c < 2; ++c) sum[c] += __shfl_xor_sync(0xFFFFFFFFu, sum[c], o);
 #pragma unroll
         for (int c = 0; c < 2; ++c)
-            if (lane < kFewCtas && h0 + c * kFewWarps < a.Hq)
-                st_cluster_f2(cluster_map(&s_part[rank][h0 + c * kFewWarps], lane), m[c], sum[c]);
+            if (lane < ctas && h0 + c * half < a.Hq)
+                st_cluster_f2(cluster_map(&s_part[rank * runs + run][h0 + c * half], lane), m[c], sum[c]);
     }
     cluster_arrive();
     cluster_wait();
-    static_assert(kFewCtas == 16, "half a warp merges the ranks of a head");
-    for (int x = tid; x - tid < a.Hq * kFewCtas; x += kFewThreads) {
-        const int h = x / kFewCtas;
-        const float2 part = h < a.Hq ? s_part[x % kFewCtas][h] : make_float2(-INFINITY, 0.f);
+    static_assert(kFewRuns == 16, "half a warp merges the runs of a head");
+    for (int x = tid; x - tid < a.Hq * kFewRuns; x += kFewThreads) {
+        const int h = x / kFewRuns;
+        const float2 part = h < a.Hq ? s_part[x % kFewRuns][h] : make_float2(-INFINITY, 0.f);
         float m = part.x;
 #pragma unroll
-        for (int o = kFewCtas / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+        for (int o = kFewRuns / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
         float sum = part.x > -INFINITY ? part.y * exp_factor(part.x - m) : 0.f;
 #pragma unroll
-        for (int o = kFewCtas / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-        if (h < a.Hq && x % kFewCtas == 0) {
+        for (int o = kFewRuns / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
+        if (h < a.Hq && x % kFewRuns == 0) {
             s_m[h] = m;
             s_inv[h] = 1.0f / sum;
         }
     }
     __syncthreads();
-    uint32_t* keys = reinterpret_cast<uint32_t*>(zs + static_cast<size_t>(a.Hq) * stride);
+    uint32_t* keys = reinterpret_cast<uint32_t*>(zs + static_cast<size_t>(a.Hq) * row);
     const uint32_t keys0 = cluster_map(keys, 0);
     for (int i = tid; i < len; i += kFewThreads) {
         float score = 0.f;
-        for (int h = 0; h < a.Hq; ++h) score += expf(zs[h * stride + i] - s_m[h]) * s_inv[h];
+        for (int h = 0; h < a.Hq; ++h) score += expf(zs[h * row + i] - s_m[h]) * s_inv[h];
         if (sc) sc[lo + r0 + i] = score;
         if (pick) st_cluster_u32(keys0 + 4 * (r0 + i), float_key(score));
     }
@@ -1045,52 +1043,107 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     if (tid == 0) sel_count[u] = a.k;
 }
 
-// Shared memory of k_select_few for these parameters, 0 when it does not fit
-// (or the shapes are outside it): the three kernels serve those.
-struct FewPlan {
-    int stride;
-    size_t smem;
-};
-FewPlan few_plan(const Derived& d, bool per_subchunk, int max_units)
+// Blocks of a run in shared memory, and the bytes of a rank in clusters of
+// `ctas` (0 when they do not fit).
+int few_stride(const Derived& d)
 {
-    FewPlan p{0, 0};
-    if (max_units > kFewUnits || d.g > 8 || d.Hq > kFusedMaxHeads) return p;
-    const int64_t logits = static_cast<int64_t>(d.nb) * d.Hq;
-    const int rounds = logits <= (1 << 11) ? 3 : logits <= (1 << 14) ? 2 : 1;
-    if (per_subchunk && max_units > rounds * kFewClusters) return p;
-    const int64_t stride = ((d.nb + kFewCtas - 1) / kFewCtas + 7) / 8 * 8;
-    const int64_t bytes = (stride * d.Hq + d.nb + kTopkPad) * 4;
-    if (bytes > kFewSmem - 48 * 1024) return p;
-    p.stride = static_cast<int>(stride);
-    p.smem = static_cast<size_t>(bytes);
-    return p;
+    return static_cast<int>(((d.nb + kFewRuns - 1) / kFewRuns + 7) / 8 * 8);
+}
+size_t few_smem(const Derived& d, int ctas)
+{
+    const int64_t bytes = (static_cast<int64_t>(few_stride(d)) * (kFewRuns / ctas) * d.Hq + d.nb + kTopkPad) * 4;
+    return bytes <= kFewSmem ? static_cast<size_t>(bytes) : 0;
+}
+
+// Time of one SM for a unit's candidates, in ns: the dot products and votes grow
+// with the query heads, the reads of the representatives with the KV heads.
+int64_t few_work(const Derived& d) { return d.nb * (d.Hq + 4 * d.Hkv); }
+
+// Whether the sequence's selection runs in k_select_few, whatever the range of a
+// call: the scores of k_logits and k_select_fused differ from its in the last
+// bits, and a unit must have the same scores, and so the same blocks, in a call
+// of its own and in one over the whole sequence. k_select_few is faster in
+// calls of few units (the loop over outer chunks), the other kernels over many;
+// GPU time per call, 32 heads on 8, one unit and 64 units:
+//   blocks              256          512         1024         2048         4096
+//   k_select_few     9.4  20.5   9.8  28.5   12.4  45.6   17.0  80.0   26.5  146 us
+//   the others      16.6  17.3  17.4  18.4   18.3  21.7   21.6  29.5   35.7   50 us
+// The line is where a call over the whole sequence takes about twice as long
+// (64 units of 1024 blocks); the kernels beyond kSortMax blocks are slower (8192
+// blocks: one unit 84 us against 45, 64 units 115 against 215, 256 units 252
+// against 809 us beside a layer's attention of some 100 ms).
+constexpr int64_t kFewLine = 1ll << 22;
+constexpr int64_t kFewLineLong = 1ll << 27;
+bool few_sequence(const Derived& d)
+{
+    return d.g <= 8 && d.Hq <= kFusedMaxHeads && few_smem(d, kFewRuns) > 0 &&
+           d.M * few_work(d) <= (d.nb <= kSortMax ? kFewLine : kFewLineLong);
+}
+
+// CTAs of a unit's cluster: the size with the shortest call by estimate, the
+// rounds of the clusters that run at once times 5 us and the unit's work.
+// Measured, 32 heads on 8 and 256 / 1024 blocks, clusters of 16, 8, 4, 2, 1:
+//    1 unit    9.4 / 12.3   10.5 / 16.6   13.8 / 25.9   20.4 / 44.8   33.2 / 82.7 us
+//   14 units  14.8 / 21.3   10.6 / 17.0   13.8 / 26.3   20.3 / 45.1   33.0 / 82.1
+//   36 units  35.0 / 54.7   23.6 / 41.9   14.0 / 26.6   20.4 / 45.3   33.2 / 82.3
+//   64 units  55.6 / 86.6   36.6 / 65.3   26.1 / 50.0   20.6 / 45.6   33.1 / 82.2
+int few_ctas(const Derived& d, int units)
+{
+    constexpr int kSlots[5] = {7, 14, 36, 76, 152};  // clusters of 16, 8, 4, 2, 1 at once
+    int best = 0;
+    float least = 0.f;
+    for (int i = 0; i < 5; ++i) {
+        const int ctas = kFewRuns >> i;
+        if (!few_smem(d, ctas)) break;
+        const float us = static_cast<float>((units + kSlots[i] - 1) / kSlots[i]) *
+                         (5.0f + 1e-3f * static_cast<float>(few_work(d)) / static_cast<float>(ctas));
+        if (!best || us < least) {
+            best = ctas;
+            least = us;
+        }
+    }
+    return best;
+}
+
+// Units to expect among `max_units` sub-chunks: the host does not know the
+// clusters that a threshold has closed, between one per S_max sub-chunks and one
+// each; the geometric mean of the two is off by no more than sqrt(S_max) either way.
+int few_units(const Derived& d, bool per_subchunk, int max_units)
+{
+    if (per_subchunk) return max_units;
+    const int per_outer = d.per_outer < max_units ? d.per_outer : max_units;
+    const int size = d.S_max < per_outer ? d.S_max : per_outer;
+    const float least = std::ceil(static_cast<float>(max_units) / static_cast<float>(size));
+    return static_cast<int>(d.theta <= -1.0f ? least : std::ceil(std::sqrt(least * static_cast<float>(max_units))));
 }
 
 template <int G>
-cudaError_t run_select_few(const SelArgs& a, const FewPlan& p, int max_units, const float* fp, const float* reps,
-                           float* scores, int32_t* sel, int32_t* sel_count, cudaStream_t st)
+cudaError_t run_select_few(const Derived& d, const SelArgs& a, int ctas, int max_units, const float* fp,
+                           const float* reps, float* scores, int32_t* sel, int32_t* sel_count, cudaStream_t st)
 {
+    auto kern = ctas == kFewRuns ? k_select_few<G, 1> : k_select_few<G, 0>;
     // set on every launch: the attributes belong to the current device
-    cudaError_t e = cudaFuncSetAttribute(k_select_few<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(p.smem));
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_select_few<G>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const size_t smem = few_smem(d, ctas);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess && ctas == kFewRuns)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
-    return launch_after(st, dim3(kFewCtas, static_cast<unsigned>(max_units)), kFewThreads, p.smem, kFewCtas,
-                        k_select_few<G>, a, fp, reps, p.stride, scores, sel, sel_count);
+    return launch_after(st, dim3(static_cast<unsigned>(ctas), static_cast<unsigned>(max_units)), kFewThreads, smem,
+                        ctas, kern, a, fp, reps, few_stride(d), scores, sel, sel_count);
 }
 
-cudaError_t launch_select_few(const Derived& d, const SelArgs& a, const FewPlan& p, int max_units, const float* fp,
+cudaError_t launch_select_few(const Derived& d, const SelArgs& a, int ctas, int max_units, const float* fp,
                               const float* reps, float* scores, int32_t* sel, int32_t* sel_count, cudaStream_t st)
 {
     switch (d.g) {
-    case 1: return run_select_few<1>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    case 2: return run_select_few<2>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    case 3: return run_select_few<3>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    case 4: return run_select_few<4>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    case 5: return run_select_few<5>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    case 6: return run_select_few<6>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    case 7: return run_select_few<7>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
-    default: return run_select_few<8>(a, p, max_units, fp, reps, scores, sel, sel_count, st);
+    case 1: return run_select_few<1>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    case 2: return run_select_few<2>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    case 3: return run_select_few<3>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    case 4: return run_select_few<4>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    case 5: return run_select_few<5>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    case 6: return run_select_few<6>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    case 7: return run_select_few<7>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
+    default: return run_select_few<8>(d, a, ctas, max_units, fp, reps, scores, sel, sel_count, st);
     }
 }
 
@@ -1433,14 +1486,16 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
     const int max_units = a.sc_end - a.sc_begin;  // units in range <= sub-chunks in range
     if (max_units <= 0) return cudaSuccess;
 
-    const FewPlan few = few_plan(d, a.ut.per_subchunk, max_units);
-    if (few.stride) {
-        // A cluster of 16 may not be had everywhere (a partition of the device);
-        // nothing is enqueued then and the kernels below do the work.
-        const cudaError_t ef = launch_select_few(d, a, few, max_units, fingerprints, reps, sel_scores, sel_blocks,
-                                                 sel_count, st);
-        if (ef == cudaSuccess) return ef;
-        cudaGetLastError();
+    if (few_sequence(d)) {
+        // A large cluster may not be had everywhere (a partition of the device);
+        // nothing is enqueued then and a smaller one does the same work, or the
+        // kernels below where its share does not fit.
+        for (int ctas = few_ctas(d, few_units(d, a.ut.per_subchunk, max_units)); ctas && few_smem(d, ctas); ctas /= 2) {
+            const cudaError_t ef = launch_select_few(d, a, ctas, max_units, fingerprints, reps, sel_scores, sel_blocks,
+                                                     sel_count, st);
+            if (ef == cudaSuccess) return ef;
+            cudaGetLastError();
+        }
     }
     // Tiles per CTA: as many as leave every SM a CTA, at most kLtSeg.
     int sms = 0;

@@ -1,9 +1,9 @@
-"""Block-level selection against the same rule in 64 bits, at the sizes where the few-unit kernel's
-runs, groups and cluster end and on both sides of the line to the kernels for many units.
+"""Block-level selection against the same rule in 64 bits, at the sizes where the one-launch kernel's
+runs, groups and clusters end and on both sides of the line to the kernels for sequences of more work.
 
 Scores: the error of a logit is the relative error of the score. The tensor-core kernel adds 48 partial
 products per logit into an fp32 accumulator, each addition off by at most 2^-23 (truncation) of a partial
-sum, taken as at most the largest logit: 48 * 2^-23 * max|z|. The few-unit kernel's fp32 sums of 128
+sum, taken as at most the largest logit: 48 * 2^-23 * max|z|. The one-launch kernel's fp32 sums of 128
 products in trees stay far below that. A selection may differ only by blocks whose score is that close to
 the k-th one; equal representatives give bit-equal scores, so exact ties have to go to the lower block.
 """
@@ -21,7 +21,7 @@ PER_SUB = S.SCALE_MODE_PER_SUBCHUNK
 # (query heads, KV heads, tokens, sub-chunk, block, sinks, window, k, units of the call, repeated rows)
 CASES = [
     (4, 1, 1100, 64, 8, 0, 0, 1, 16, False),
-    (4, 1, 1100, 64, 8, 0, 0, 1, 18, False),        # one more unit than a call of the few-unit kernel
+    (4, 1, 1100, 64, 8, 0, 0, 1, 18, False),        # clusters of 4 CTAs
     (1, 1, 4000, 1000, 3, 5, 17, 100, 4, True),     # ragged blocks, exact ties across the ranks
     (2, 1, 4000, 1000, 16, 16, 100, 249, 4, False),  # k = candidates - 1 and candidates for some units
     (3, 1, 5000, 500, 7, 40, 100, 33, 9, False),
@@ -29,17 +29,23 @@ CASES = [
     (12, 2, 5000, 1000, 9, 0, 1, 64, 5, False),
     (28, 4, 8200, 1024, 33, 64, 128, 20, 9, False),
     (64, 8, 8200, 1024, 64, 64, 128, 20, 8, True),
-    (256, 64, 3000, 1000, 64, 64, 128, 8, 3, False),  # the most heads of the fused kernels
+    (256, 64, 3000, 1000, 64, 64, 128, 8, 3, False),  # the most heads of the one-launch kernel
     (260, 52, 3000, 1000, 64, 64, 128, 8, 3, False),  # and beyond
-    (10, 1, 3000, 1000, 32, 0, 0, 8, 3, False),       # group of 10: the kernels for many units
+    (10, 1, 3000, 1000, 32, 0, 0, 8, 3, False),       # group of 10: the other kernels
     (4, 1, 40000, 10000, 10, 0, 0, 4000, 4, False),   # 4000 blocks
-    (32, 8, 70000, 10000, 16, 64, 128, 1000, 7, True),  # more blocks than the shared memory holds
+    (32, 8, 70000, 10000, 16, 64, 128, 1000, 7, True),  # more than 4096 blocks
     (4, 2, 3000, 1000, 64, 64, 128, 0, 3, False),     # nothing selected
     (4, 1, 300000, 10000, 64, 64, 1024, 64, 30, True),  # many units, 4,688 blocks
-    (32, 8, 16416, 1000, 32, 0, 0, 64, 7, True),     # 513 x 32 logits a unit: one round of clusters
-    (32, 8, 16416, 1000, 32, 0, 0, 64, 8, True),     # and one unit more
-    (32, 8, 16384, 1024, 32, 0, 0, 64, 14, False),   # 2^14: two rounds
+    (32, 8, 16416, 1000, 32, 0, 0, 64, 7, True),     # the most units of clusters of 16
+    (32, 8, 16416, 1000, 32, 0, 0, 64, 8, True),     # and one unit more: clusters of 8
+    (32, 8, 16384, 1024, 32, 0, 0, 64, 14, False),   # the most units of those
     (32, 8, 16384, 1024, 32, 0, 0, 64, 15, False),
+    # the kernels for sequences of more work: 16-byte and 4-byte loads, segments of several unit tiles
+    (32, 8, 66000, 500, 64, 64, 128, 20, 9, True),     # 1,032 blocks
+    (28, 4, 66000, 300, 61, 40, 100, 33, 15, False),   # 1,082 blocks
+    (8, 8, 66000, 220, 64, 0, 1, 64, 300, True),
+    (256, 64, 6400, 64, 64, 64, 128, 8, 4, False),
+    (10, 1, 40000, 10000, 9, 0, 0, 300, 4, True),      # more than 4096 blocks
 ]
 
 
