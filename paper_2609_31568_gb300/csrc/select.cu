@@ -749,9 +749,10 @@ __global__ void __launch_bounds__(kTopkThreads) k_topk(SelArgs a, const float* _
 // Steps (b)-(c) after the logits for units of at most kSortMax candidates,
 // one CTA of kTopkThreads per unit: the heads' statistics, the soft vote
 // (scores written where asked for, NaN off the candidates) and the short path
-// of k_topk. A warp takes a head's statistics in one pass (each lane a running
-// reference, raised when a logit outgrows it by 8, and the sum of exp(z -
-// reference)); both passes over the logits load VEC blocks at a time, which is
+// of k_topk. A warp takes a head's statistics in one pass (each lane the running
+// maximum and the sum of exp(z - maximum), so the large terms take no rounding
+// of the exponential's argument: raised only by jumps of 8, the errors of rows
+// of standard deviation 8 to 12 were up to 9 % larger); both passes over the logits load VEC blocks at a time, which is
 // what bounds the kernel: latency times the bytes in flight. 256 units of up to
 // 4,096 blocks and 32 heads: 34 us (scalar loads, max and sum in two
 // passes: 51 us). VEC is 4 where the rows allow 16-byte loads.
@@ -810,7 +811,7 @@ __global__ void __launch_bounds__(kTopkThreads) k_select_fused(SelArgs a, const 
                 for (int i = 0; i < kIn; ++i)
 #pragma unroll
                     for (int c = 0; c < VEC; ++c) top = fmaxf(top, x[i][c]);
-                if (top > m + 8.0f) {
+                if (top > m) {
                     sum *= exp_factor(m - top);
                     m = top;
                 }

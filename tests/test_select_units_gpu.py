@@ -101,3 +101,38 @@ def test_block_selection_of_units(hq, hkv, n, sub, block, sink, local, k, units,
                     for r in torch.unique((one - lo) % 61):
                         mine = got[(got - lo) % 61 == r]
                         assert torch.equal(mine, torch.arange(len(mine), device="cuda") * 61 + r + lo)
+
+
+@pytest.mark.parametrize("nb,batch", [(2064, 1024), (2062, 256)])  # 16-byte and 4-byte loads
+def test_large_terms_are_summed_against_their_maximum(nb, batch):
+    """A head whose probability lies on 32 equal blocks, met by the lanes of a warp after blocks 6 to 8 below
+    them (by lane 0 before): the large terms of its sum are exactly 1, as in a sum over the known maximum.
+    What is left in the root mean square over 64 gaps is the rounding of a lane's sum (2^-24 / sqrt(3)), the
+    reciprocal (an ulp: 2^-23 / sqrt(3)) and the additions over the lanes, of nearly equal values and so
+    nearly exact: 8e-8, and half as much again for them (measured 4e-8). Terms taken against a reference 6
+    to 8 below them carry the rounding of an argument of 8 to 12 log2 units as well: 1.6e-7."""
+    lane = torch.arange(32, device="cuda") * (4 if nb % 4 == 0 else 1)
+    block, sub = 2, 8
+    n = nb * block
+    m = -(-n // sub)
+    reps = torch.zeros(1, nb, 128, device="cuda")
+    reps[0, :, 1] = -200.0
+    low, high = lane.clone(), lane + batch
+    low[0], high[0] = batch, 0
+    reps[0, low, :2] = 0.0
+    reps[0, high, 0], reps[0, high, 1] = 7.875, 0.0
+    fp = torch.zeros(m, 128, device="cuda")
+    fp[:, 0] = 0.75 + (torch.arange(m, device="cuda") % 64 + 1) / 256  # the gap / 7.875; exact logits
+    fp[:, 1] = 1.0
+    p = S.params(num_q_heads=1, num_kv_heads=1, sub_chunk=sub, n_tokens=n, max_cluster_subchunks=1, block_size=block,
+                 top_k=8, n_sink=0, n_local=0)
+    buf = pkg.allocate(p, PER_SUB, want_scores=True)
+    S.scale_select(p, PER_SUB, 0, n, reps, fp, None, None, buf.sel_blocks, buf.sel_count, buf.sel_scores, buf.ws)
+    torch.cuda.synchronize()
+    rel = []
+    for u in range(m - 64, m):
+        z = fp[u, 0].double() * reps[0, : u * sub // block, 0].double() + reps[0, : u * sub // block, 1].double()
+        ref = torch.softmax(z, 0)[high]
+        rel.append(((buf.sel_scores[u][high].double() - ref) / ref).mean())
+    rms = float(torch.stack(rel).square().mean().sqrt())
+    assert rms < 1.2e-7, rms
