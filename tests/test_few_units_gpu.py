@@ -90,6 +90,34 @@ def test_few_unit_token_selection(hq, hkv, n, sub, sink, local, k, ties):
                 assert _near(got[:count], want, ref, sink, 2e-5)
 
 
+@pytest.mark.parametrize("n,spread", [(16384, 2.0), (100003, 2.0), (100003, 3.0), (100003, 8.0)])
+def test_error_of_spread_logits(n, spread):
+    """Exact logits (a coordinate of a bf16 key each): what is left of a score's error is the exponential's,
+    two ulps at most and less than one in the root mean square, and the rounding of its argument, a
+    difference of at most a few units for the tokens that carry the score: 2^-24 8 ln 2 / sqrt(3) for the
+    largest of them. 1e-7 together, 1.6e-7 with a margin; with the product of logit and scale rounded
+    before the difference and references between which the factors are approximate 1.7e-7 to 3.2e-7."""
+    sub = 1024
+    m = -(-n // sub)
+    rel = []
+    for seed in range(8):
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        keys = torch.zeros(n, 1, 128, dtype=torch.bfloat16, device="cuda")
+        keys[:, 0, :8] = spread * torch.randn(n, 8, generator=gen, device="cuda")
+        fp = torch.eye(8, 128, device="cuda").flatten().repeat(m, 1)
+        p = S.params(num_q_heads=8, num_kv_heads=1, sub_chunk=sub, n_tokens=n, max_cluster_subchunks=1,
+                     block_size=1, top_k=2048, n_sink=0, n_local=0)
+        buf = pkg.allocate(p, PER_SUB, want_scores=True)
+        S.scale_select_tokens(p, PER_SUB, (m - 4) * sub, n, keys, fp, None, None, buf.sel_blocks, buf.sel_count,
+                              buf.sel_scores, buf.ws)
+        torch.cuda.synchronize()
+        for u in range(m - 4, m):
+            ref = torch.softmax(keys[: u * sub, 0, :8].double(), 0).sum(1)
+            rel.append(float((buf.sel_scores[u, : u * sub].double() - ref).norm() / ref.norm()))
+    mean = sum(rel) / len(rel)
+    assert mean < 1.6e-7, mean
+
+
 def _near(got, want, ref, sink, rel):
     """Whether every token in only one of the lists scores within `rel` of the k-th score."""
     kth = ref[want - sink].min()
