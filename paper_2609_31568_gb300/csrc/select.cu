@@ -923,7 +923,7 @@ __global__ void __launch_bounds__(kFewThreads, 1) k_select_few(SelArgs a, const 
     using namespace scale_ptx;
     constexpr int NB = G <= 4 ? 8 : 4;
     constexpr int V = G == 1 ? 8 : G == 2 ? 16 : 32;
-    extern __shared__ float zs[];
+    extern __shared__ __align__(16) float zs[];  // topk_emit reads the keys behind them 16 bytes at a time
     __shared__ float2 s_part[kFewRuns][kFusedMaxHeads + 1];  // + 1: a head's runs in different banks
     __shared__ float s_m[kFusedMaxHeads], s_inv[kFusedMaxHeads];
     __shared__ TopkShared sh;
