@@ -181,8 +181,11 @@ def _stream(stream) -> int | None:
             import torch
 
             _torch = torch
-        # the handle alone: 0.3 us, against 3 us for a torch.cuda.Stream object
-        return _torch._C._cuda_getCurrentRawStream(_torch.cuda.current_device())
+        # the handle alone, where this torch gives it: 0.3 us, against 3 us for a torch.cuda.Stream object
+        raw = getattr(_torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            return _torch.cuda.current_stream().cuda_stream
+        return raw(_torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

@@ -39,6 +39,19 @@ def test_wait_limit_entry_points_validate(lib):
     assert lib.scale_selftest_wait_timeout(None, 0, 1_000_000, None) == S.SCALE_ERR_INVALID_ARG
 
 
+def test_current_stream_without_the_private_handle(monkeypatch):
+    """A torch that lacks the private function for the raw handle gives the stream through its public call."""
+    from types import SimpleNamespace
+
+    cuda = SimpleNamespace(current_stream=lambda: SimpleNamespace(cuda_stream=1234), current_device=lambda: 3)
+    monkeypatch.setattr(S, "_torch", SimpleNamespace(_C=SimpleNamespace(), cuda=cuda))
+    assert S._stream(None) == 1234
+    handle = SimpleNamespace(_cuda_getCurrentRawStream=lambda device: 100 + device)
+    monkeypatch.setattr(S, "_torch", SimpleNamespace(_C=handle, cuda=cuda))
+    assert S._stream(None) == 103
+    assert S._stream(7) == 7 and S._stream(SimpleNamespace(cuda_stream=8)) == 8
+
+
 def test_params_struct_layout_matches_header():
     src = r"""
 #include <stddef.h>
