@@ -84,46 +84,30 @@ def load_peaks():
 
 
 def launches(w, selects: int = 1, builds: int = 1) -> dict:
-    """Kernels of the path's steps for workload w with `builds` step-(a) calls and
-    `selects` select + attend calls, every step a kernel of its own (block size
-    1 skips the representatives, scores in four kernels and gathers the distant
-    keys through a per-unit list). `issued_launches` counts what is launched:
-    steps that share a kernel once."""
-    tok = w.block_size == 1
-    build = (2 if tok else 3) + (1 if w.max_cluster_subchunks > 1 else 0)
-    # the top-k is one kernel, or 8 (init, 4 histogram passes, count, scan,
-    # emit) for units of more than 64K candidates
-    topk = 8 if tok and w.n_blocks > 65536 else 1
-    if tok:
-        select = 4 + topk
-    else:
-        # logits, then statistics + vote + top-k in one kernel up to 4096 blocks
-        select = 2 if w.n_blocks <= 4096 and w.num_q_heads <= 256 else 3 + topk
-    attend = 3 if tok else 1
-    return {"build_reps": build * builds, "select": select * selects, "attend": attend * selects,
-            "total": build * builds + (select + attend) * selects}
-
-
-def issued_launches(w, selects: int = 1, builds: int = 1) -> dict:
-    """Kernel launches of the library for the same calls: step (a) is one kernel,
-    and a second where a threshold decides the clusters; a selection call of at
-    most 16 sub-chunks is one kernel at block level (if its logits fit shared
-    memory) and three at token level (if its planes of logits fit the workspace)."""
-    tok = w.block_size == 1
+    """Kernel launches of the library for workload w with `builds` step-(a) calls and `selects` select +
+    attend calls. Step (a) is one kernel, and a second where a threshold decides the clusters. Block-level
+    selection is one kernel for sequences of little selection work, two (logits; statistics, vote and top-k)
+    up to 4096 blocks, else four. Token-level selection is three kernels for calls of at most 16 sub-chunks
+    whose planes of logits fit the workspace, else four and the top-k (eight beyond 65,536 candidates), and
+    its attention gathers the distant keys in two kernels of its own."""
     per_call = -(-w.n_subchunks // selects)
     build = 2 if w.max_cluster_subchunks > 1 and w.theta > -1.0 else 1
-    few = per_call <= 16 and w.group <= 8
-    if tok:
+    if w.block_size == 1:
         slots = -(-(w.n_sink + w.top_k) // 128) * 128
         room = 2 * w.n_subchunks * w.num_kv_heads * slots * 256
         scratch = -(-per_call * (3 * 2048 + 16 + 512) * 4 // 256) * 256
-        few = few and scratch + per_call * w.num_q_heads * (-(-w.n_tokens // 4) * 4) * 4 <= room
-        select = 3 if few else 4 + (8 if w.n_blocks > 65536 else 1)
+        planes = per_call * w.num_q_heads * (-(-w.n_tokens // 4) * 4) * 4
+        select = 3 if per_call <= 16 and scratch + planes <= room else 4 + (8 if w.n_blocks > 65536 else 1)
+        attend = 3
     else:
-        stride = -(-(-(-w.n_blocks // 16)) // 8) * 8
-        few = few and w.num_q_heads <= 256 and (stride * w.num_q_heads + w.n_blocks + 128) * 4 <= 152 * 1024
-        select = 1 if few else 2 if w.n_blocks <= 4096 and w.num_q_heads <= 256 and w.top_k <= 4096 else 4
-    attend = 3 if tok else 1
+        run = -(-(-(-w.n_blocks // 16)) // 8) * 8
+        work = w.n_subchunks * w.n_blocks * (w.num_q_heads + 4 * w.num_kv_heads)
+        if (w.group <= 8 and w.num_q_heads <= 256 and (run * w.num_q_heads + w.n_blocks + 128) * 4 <= 152 * 1024
+                and work <= (1 << 22 if w.n_blocks <= 4096 else 1 << 27)):
+            select = 1
+        else:
+            select = 2 if w.n_blocks <= 4096 and w.num_q_heads <= 256 and w.top_k <= 4096 else 4
+        attend = 1
     return {"build_reps": build * builds, "select": select * selects, "attend": attend * selects,
             "total": build * builds + (select + attend) * selects}
 
@@ -573,7 +557,7 @@ def run_scale(args):
         return {"ms_per_step": total, "tokens_per_s": w.n_tokens / (total / 1e3),
                 "stages_ms": {"build_reps": stages[0], "select": stages[1], "sparse_attention": stages[2]},
                 "build_calls": len(plan), "select_attend_calls": n_calls,
-                "gpu_launches": issued_launches(w, n_calls, len(plan))["total"]}, clk
+                "gpu_launches": launches(w, n_calls, len(plan))["total"]}, clk
 
     def unit_stats(mode_, buf_):
         sub = mode_ == S.SCALE_MODE_PER_SUBCHUNK
@@ -1016,7 +1000,7 @@ def run_stack(args):
             units += n
             calls += S.scale_retrieval_calls(p, mode, None if per_sub else us[: n + 1], n)[1]
         del bufs
-        launch_count = w.layers * issued_launches(w, n_attn // w.layers, len(plan))["total"]
+        launch_count = w.layers * launches(w, n_attn // w.layers, len(plan))["total"]
         return ms, attn_ms, clk, 4.0 * w.head_dim * w.num_q_heads * keys, calls, units, launch_count, n_attn
 
     mode = S.SCALE_MODE_PER_SUBCHUNK if args.mode == "subchunk" else S.SCALE_MODE_PER_CLUSTER

@@ -67,23 +67,34 @@ def test_selection_agreement_counts():
 
 
 def test_launch_counts():
-    # step (a): k_block_reps, k_fingerprint, k_cluster (+ k_gram when clusters have > 1 sub-chunk);
-    # selection: k_logits + k_select_fused (up to 4096 blocks); attention: k_sparse_attn
-    assert bench.launches(workload("llama8b-128k"))["total"] == 7   # 4 + 2 + 1
-    assert bench.launches(workload("gqa4-4k", max_cluster_subchunks=1))["total"] == 6
-    # more than 4096 blocks: k_logits, k_stats, k_vote, k_topk
-    assert bench.launches(workload("llama8b-1m", block_size=128))["total"] == 4 + 4 + 1
-    # token level: split, two scoring passes and their merge, then the multi-CTA top-k
-    # (init, 4 histogram passes, count, scan, emit)
-    assert bench.launches(workload("llama8b-128k-tok"))["total"] == 3 + 4 + 8 + 3
-    assert bench.launches(workload("llama8b-32k", block_size=1, top_k=1024))["total"] == 3 + 5 + 3
-    # the 1M-token step of Algorithm 2: 16 outer chunks, one unit each (the ncu launch list of that step
-    # counted 288 launches of the library's kernels)
+    # step (a): k_step_a, and k_gram where a threshold decides clusters of more than one sub-chunk;
+    # selection: k_select_few, or k_logits + k_select_fused; attention: k_sparse_attn
+    w = workload("llama8b-128k")  # 64 sub-chunks of 1,024 blocks: the last sequence of k_select_few
+    assert bench.launches(w) == {"build_reps": 1, "select": 1, "attend": 1, "total": 3}
+    assert bench.launches(w, 8, 8)["total"] == 8 * 3  # the loop over outer chunks
+    assert bench.launches(w, 64, 8)["total"] == 8 + 64 * 2  # a call per sub-chunk
+    assert bench.launches(w.replace(n_tokens=w.n_tokens + 1))["select"] == 2
+    assert bench.launches(w.replace(n_tokens=w.n_tokens + 1), 8)["select"] == 16
+    assert bench.launches(w.replace(theta=0.9))["build_reps"] == 2
+    assert bench.launches(w.replace(theta=0.9, max_cluster_subchunks=1))["build_reps"] == 1
+    # 4096 blocks and beyond: k_logits, k_stats, k_vote, k_topk
+    w = workload("llama8b-1m")
+    assert w.n_blocks == 4096 and bench.launches(w)["select"] == 2
+    assert bench.launches(w.replace(block_size=128))["select"] == 1  # 8,192 blocks, 2^27 at most
+    assert bench.launches(w.replace(block_size=64))["select"] == 4
+    # token level: k_tok_split, k_key_logits and k_vote_topk for at most 16 sub-chunks, else k_tok_split, two
+    # scoring passes and their merge, and the top-k of many candidates (init, 4 histogram passes, count, scan,
+    # emit) or of few; k_tok_lists and k_tok_pack before the attention
     w = workload("llama8b-1m-tok")
     chunks = w.n_tokens // w.outer_chunk
-    assert bench.launches(w, chunks, chunks)["total"] == 288
-    assert bench.launches(workload("llama8b-64k-32l"), 8)["total"] == 4 + 8 * 3
-    assert bench.launches(workload("llama8b-64k-32l"), 8, 8)["total"] == 8 * 4 + 8 * 3  # per-chunk step (a)
+    assert bench.launches(w, chunks, chunks)["total"] == 16 * (1 + 3 + 3)
+    assert bench.launches(w)["select"] == 4 + 8
+    assert bench.launches(workload("llama8b-32k", block_size=1, top_k=1024), 2)["select"] == 2 * 3
+    assert bench.launches(workload("llama8b-32k", block_size=1, top_k=1024))["select"] == 4 + 1
+    # planes of 4 H_q N bytes per sub-chunk of the call in 512 M H_kv (sinks + k) bytes: seven fit
+    w = workload("llama8b-1m-tok", top_k=896)
+    assert bench.launches(w, 64)["select"] == 64 * 3
+    assert bench.launches(w, 32)["select"] == 32 * (4 + 8)
 
 
 def test_other_configs_compacts_each_side_run(monkeypatch):
