@@ -182,7 +182,8 @@ int scale_build_reps_noalloc(const scale_params_t *p, const void *q, const void 
  * |candidates|). tok_begin and tok_end must be multiples of outer_chunk (SCR)
  * or sub_chunk (baseline), or tok_end == N.
  *   sel_scores  fp32 [M][nb] or NULL: score_b on the candidates, NaN elsewhere.
- * unit_start / n_units are ignored in baseline mode (may be NULL). */
+ * unit_start / n_units are ignored in baseline mode (may be NULL). A unit's
+ * scores and blocks are the same, bit for bit, in whichever range call it is. */
 int scale_select(const scale_params_t *p, int32_t mode, int64_t tok_begin, int64_t tok_end,
                  const float *reps, const float *fingerprints, const int32_t *unit_start,
                  const int32_t *n_units, int32_t *sel_blocks, int32_t *sel_count,
@@ -201,7 +202,11 @@ int scale_select(const scale_params_t *p, int32_t mode, int64_t tok_begin, int64
  *   sel_tokens  int32 [M][top_k] out (ascending token indices, -1 padded)
  *   sel_count   int32 [M] out
  *   sel_scores  fp32 [M][N] or NULL: score_t on the candidates, NaN elsewhere.
- * Same range rule, modes and workspace as scale_select. H_q / H_kv must be at
+ * Same range rule, modes and workspace as scale_select. The last bits of a
+ * unit's scores depend on the other units of its call and on its range (about
+ * 1e-7 of a score): of tokens whose scores are that close to the k-th one, two
+ * calls may pick different ones. Equal keys have bit-equal scores in a call.
+ * H_q / H_kv must be at
  * most 8 (SCALE_ERR_UNSUPPORTED otherwise); block_size != 1 gives
  * SCALE_ERR_INVALID_ARG (and scale_select gives SCALE_ERR_UNSUPPORTED for
  * block size 1). */
@@ -336,8 +341,9 @@ int scale_retrieval_calls(const scale_params_t *p, int32_t mode, const int32_t *
  * have arrived, while the next piece's rows are copied in and the previous
  * piece's output is copied out on two streams of the call's own. When L or
  * n_local is not a multiple of 128 it runs as one piece. The result equals the
- * whole-sequence calls bit for bit. The call creates and releases those
- * streams and their events itself. */
+ * whole-sequence calls bit for bit; at block size 1 for the same selection (see
+ * scale_select_tokens). The call creates and releases those streams and their
+ * events itself. */
 int scale_prefill_host_arena_size(const scale_params_t *p, int32_t mode, size_t *bytes);
 int scale_prefill_host(const scale_params_t *p, int32_t mode, const void *q_host,
                        const void *k_host, const void *v_host, void *out_host, void *arena,
