@@ -102,7 +102,9 @@ typedef struct scale_params {
 } scale_params_t;
 
 /* Bytes of workspace that scale_build_reps / scale_select / scale_sparse_prefill
- * need for `p` and `mode` (one workspace serves all three). Synchronous, host only. */
+ * need for `p` and `mode` (one workspace serves all three). Calls that share a
+ * workspace must not overlap on the GPU: a selection at block size 1 keeps its
+ * logits where an attention call keeps its packed keys. Synchronous, host only. */
 int scale_workspace_size(const scale_params_t *p, int32_t mode, size_t *bytes);
 
 /* Zero the workspace header (the device status word). Call once after
@@ -350,7 +352,7 @@ int scale_prefill_host(const scale_params_t *p, int32_t mode, const void *q_host
                        size_t arena_bytes, scale_stream_t stream);
 
 /* Upper bound, in nanoseconds of wall time, of every device-side wait of the
- * attention kernel (default 4e9). A wait that runs out records
+ * selection, attention and decode kernels (default 4e9). A wait that runs out records
  * SCALE_ERR_TIMEOUT in the device status and the kernel returns. Process-wide;
  * applies to launches issued after the call. ns = 0 is refused with
  * SCALE_ERR_INVALID_ARG and leaves the limit unchanged. */
