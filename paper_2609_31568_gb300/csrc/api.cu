@@ -589,7 +589,7 @@ int scale_decode_workspace_size(const scale_params_t* p, size_t* bytes)
     int rc = derive(p, &d);
     if (rc) return rc;
     if (!bytes) return SCALE_ERR_INVALID_ARG;
-    *bytes = decode_ws_bytes(d, decode_splits());
+    *bytes = decode_ws_bytes(d);
     return SCALE_OK;
 }
 
@@ -606,7 +606,7 @@ int scale_decode_step(const scale_params_t* p, int64_t t, const void* q_t, const
     if (!device_ptr(q_t, 16) || !device_ptr(k, 16) || !device_ptr(v, 16) || !device_ptr(out_t, 16) ||
         !device_ptr(cache, 256) || !device_ptr(ws, 256))
         return SCALE_ERR_INVALID_ARG;
-    if (cache_bytes < decode_cache_bytes(d) || ws_bytes < decode_ws_bytes(d, decode_splits()))
+    if (cache_bytes < decode_cache_bytes(d) || ws_bytes < decode_ws_bytes(d))
         return SCALE_ERR_WORKSPACE;
     return cuda_status(launch_decode_step(d, t, q_t, k, v, static_cast<uint8_t*>(cache), out_t,
                                           static_cast<uint8_t*>(ws), g_timeout_ns.load(), stream));

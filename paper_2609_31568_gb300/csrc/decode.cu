@@ -52,8 +52,7 @@ __device__ __forceinline__ uint4 ld_nc(const uint4* p)
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
-constexpr int kDecSlots = 128;     // partial slots per head the workspace is sized for
-constexpr int kDecMaxSplits = 64;  // of which the attention kernel uses at most these
+constexpr int kDecMaxSplits = 64;  // key splits of a KV head
 // Threads of an attention CTA: one CTA of 512 per SM where a thread's 128
 // registers hold its G query heads, else 256. Half as many CTAs of twice the
 // size leave half the partials for the CTA that merges them.
@@ -333,8 +332,45 @@ cudaError_t run_dec_attn(const DecArgs& a, const void* q, const void* k, const v
                         static_cast<const uint4*>(v), static_cast<__nv_bfloat16*>(out));
 }
 
-// Chunks of 64 keys that the workspace holds a (max, sum) pair for.
+// Keys per (max, sum) pair of the logits that the workspace has room for.
 constexpr int kDecStat = 64;
+
+// Regions of the decode workspace (byte offsets from its base; the status word
+// comes first).
+struct DecWs {
+    size_t z;        // fp32 [H_q][z_stride]               logits, rows padded to four tokens
+    size_t zpart;    // float2 [H_q][n_stat]               partial softmax sums of the logits
+    size_t o_part;   // float4 [H_q][kDecMaxSplits][32]    attention: unnormalised outputs
+    size_t ml_part;  // float2 [H_q][kDecMaxSplits]        (max, sum)
+    size_t tickets;  // int32 [H_kv]
+    size_t gate;     // int32 [1]
+    size_t scratch;  // int32 [kVoteScratchInts]           vote and top-k
+    size_t end;
+    int64_t z_stride, n_stat;
+};
+
+DecWs decode_layout(const Derived& d)
+{
+    DecWs w{};
+    size_t off = 256;
+    auto take = [&](size_t bytes) {
+        const size_t at = off;
+        off = align_up(off + bytes, kAlign);
+        return at;
+    };
+    const size_t heads = static_cast<size_t>(d.Hq);
+    w.z_stride = (d.N + 3) / 4 * 4;
+    w.n_stat = (d.N + kDecStat - 1) / kDecStat;
+    w.z = take(heads * w.z_stride * sizeof(float));
+    w.zpart = take(heads * w.n_stat * sizeof(float2));
+    w.o_part = take(heads * kDecMaxSplits * kHeadDim * sizeof(float));
+    w.ml_part = take(heads * kDecMaxSplits * sizeof(float2));
+    w.tickets = take(static_cast<size_t>(d.Hkv) * sizeof(int32_t));
+    w.gate = take(sizeof(int32_t));
+    w.scratch = take(kVoteScratchInts * sizeof(int32_t));
+    w.end = off;
+    return w;
+}
 
 }  // namespace
 
@@ -344,23 +380,22 @@ size_t decode_cache_bytes(const Derived& d)
            static_cast<size_t>(d.k > 0 ? d.k : 1) * sizeof(int32_t) + 256;
 }
 
-size_t decode_ws_bytes(const Derived& d, int splits)
+// The size that callers are told, and may have stored: more than the regions
+// take (65 KB a head beside the logits and their sums, of which they take less
+// than half, and 27 KB once).
+size_t decode_ws_bytes(const Derived& d)
 {
-    const size_t cap = static_cast<size_t>(d.N);
-    size_t off = 0;
-    off = align_up(off + 256, kAlign);                                           // status word
-    off = align_up(off + static_cast<size_t>(d.Hq) * cap * sizeof(float), kAlign);  // z
-    off = align_up(off + static_cast<size_t>(d.Hq) * sizeof(float2), kAlign);   // stats
-    off = align_up(off + cap * sizeof(float), kAlign);                          // scores
-    off = align_up(off + static_cast<size_t>(d.Hq) * splits * 130 * sizeof(float), kAlign);
-    off = align_up(off + static_cast<size_t>(d.Hq) * ((cap + kDecStat - 1) / kDecStat) * sizeof(float2), kAlign);  // zpart
-    off = align_up(off + (kTopkPasses * 256 + (kTopkPasses + 1) * 4) * sizeof(int32_t), kAlign);  // top-k hist, state
-    off = align_up(off + static_cast<size_t>(topk_max_chunks(d)) * sizeof(int2), kAlign);          // top-k counts
-    return off;
+    constexpr size_t kHeadBytes = 128 * 130 * sizeof(float);
+    const size_t cap = static_cast<size_t>(d.N), heads = static_cast<size_t>(d.Hq);
+    size_t off = 256;
+    for (const size_t bytes : {heads * cap * sizeof(float), heads * sizeof(float2), cap * sizeof(float), heads * kHeadBytes,
+                               heads * ((cap + kDecStat - 1) / kDecStat) * sizeof(float2),
+                               (kTopkPasses * 256 + (kTopkPasses + 1) * 4) * sizeof(int32_t),
+                               static_cast<size_t>(topk_max_chunks(d)) * sizeof(int2)})
+        off = align_up(off + bytes, kAlign);
+    const size_t end = decode_layout(d).end;
+    return off > end ? off : end;
 }
-
-
-int decode_splits() { return kDecSlots; }
 
 cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const void* k, const void* v,
                                uint8_t* cache, void* out, uint8_t* ws, uint64_t timeout_ns, cudaStream_t st)
@@ -370,24 +405,11 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     auto* sel = reinterpret_cast<int32_t*>(cache + kDecAnchor + static_cast<size_t>(d.Hq) * kHeadDim * sizeof(float));
     int32_t* sel_count = sel + (d.k > 0 ? d.k : 1);
     auto* status = reinterpret_cast<int32_t*>(ws + kStatusOffset);
-    size_t off = 256;
-    auto take = [&](size_t bytes) {
-        const size_t at = off;
-        off = align_up(off + bytes, kAlign);
-        return at;
-    };
-    const size_t cap = static_cast<size_t>(d.N);
-    const size_t n_stat = (cap + kDecStat - 1) / kDecStat;
-    // The planes of logits, their rows padded to four tokens; the padding (at
-    // most 12 bytes per head) runs into the regions behind them, which hold
-    // nothing before the attention.
-    auto* z = reinterpret_cast<float*>(ws + take(static_cast<size_t>(d.Hq) * cap * sizeof(float)));
-    take(static_cast<size_t>(d.Hq) * sizeof(float2));
-    take(cap * sizeof(float));
-    const int64_t z_stride = (d.N + 3) / 4 * 4;
-    // the attention's partials, the tickets and the gate, the scratch of the selection
-    uint8_t* parts = ws + take(static_cast<size_t>(d.Hq) * kDecSlots * 130 * sizeof(float));
-    auto* zpart = reinterpret_cast<float2*>(ws + take(static_cast<size_t>(d.Hq) * n_stat * sizeof(float2)));
+    const DecWs lay = decode_layout(d);
+    auto* z = reinterpret_cast<float*>(ws + lay.z);
+    auto* zpart = reinterpret_cast<float2*>(ws + lay.zpart);
+    auto* gate = reinterpret_cast<int32_t*>(ws + lay.gate);
+    auto* scratch = reinterpret_cast<int32_t*>(ws + lay.scratch);
 
     DecArgs a;
     a.Hq = d.Hq;
@@ -402,16 +424,10 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     a.anchor = anchor;
     a.sel = sel;
     a.sel_count = sel_count;
-    a.o_part = reinterpret_cast<float4*>(parts);
-    a.ml_part = reinterpret_cast<float2*>(parts + static_cast<size_t>(d.Hq) * kDecMaxSplits * kHeadDim * sizeof(float));
-    a.tickets = reinterpret_cast<int32_t*>(a.ml_part + static_cast<size_t>(d.Hq) * kDecMaxSplits);
-    int32_t* gate = a.tickets + d.Hkv;
+    a.o_part = reinterpret_cast<float4*>(ws + lay.o_part);
+    a.ml_part = reinterpret_cast<float2*>(ws + lay.ml_part);
+    a.tickets = reinterpret_cast<int32_t*>(ws + lay.tickets);
     a.gate = gate;
-    auto* scratch = reinterpret_cast<int32_t*>(parts + align_up(reinterpret_cast<uint8_t*>(gate + 1) - parts, 16));
-    static_assert(kDecMaxSplits * (kHeadDim + 2) * sizeof(float) + 2 * sizeof(int32_t) + 16 +
-                          kVoteScratchInts * sizeof(int32_t) <=
-                      kDecSlots * 130 * sizeof(float),
-                  "partials, tickets and scratch of one head fit its slots");
 
     // One unit of one token, its position t (per-sub-chunk units with L = 1).
     const Units ut{nullptr, nullptr, 1, d.N, 1, static_cast<int>(d.N)};
@@ -426,7 +442,7 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     s.n_local = d.n_local;
     s.scale2 = d.sigma * 1.4426950408889634f;
     s.z = z;
-    s.z_stride = z_stride;
+    s.z_stride = lay.z_stride;
     s.part = zpart;
     s.scratch = scratch;
     s.status = status;
@@ -441,7 +457,7 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     s.tickets = a.tickets;
     const int64_t W = window_start(d.n_local, t);
     const bool any = W > d.n_sink;
-    s.n_part = any ? key_logits_parts(W - d.n_sink / 128 * 128, d.Hkv, static_cast<int64_t>(n_stat)) : 1;
+    s.n_part = any ? key_logits_parts(W - d.n_sink / 128 * 128, d.Hkv, lay.n_stat) : 1;
     cudaError_t e = launch_key_logits(s, d.g, true, q, 1, k, 1, st);
     if (e != cudaSuccess) return e;
     if (any) {
@@ -457,7 +473,7 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
         w.n_local = d.n_local;
         w.scale2 = s.scale2;
         w.z = z;
-        w.z_stride = z_stride;
+        w.z_stride = lay.z_stride;
         w.part = zpart;
         w.n_part = s.n_part;
         w.scores = nullptr;

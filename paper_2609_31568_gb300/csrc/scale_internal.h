@@ -189,8 +189,7 @@ cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, 
 int tok_range(const Derived& d);
 // Decode step (decode.cu).
 size_t decode_cache_bytes(const Derived& d);
-size_t decode_ws_bytes(const Derived& d, int splits);
-int decode_splits();
+size_t decode_ws_bytes(const Derived& d);
 cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const void* k, const void* v,
                                uint8_t* cache, void* out, uint8_t* ws, uint64_t timeout_ns, cudaStream_t st);
 
