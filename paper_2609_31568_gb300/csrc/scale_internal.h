@@ -178,8 +178,7 @@ struct TopkScratch {
 };
 int topk_max_chunks(const Derived& d);
 cudaError_t launch_topk(const Derived& d, const Units& ut, int sc_begin, int sc_end, const float* scores,
-                        int32_t* sel, int32_t* sel_count, cudaStream_t st,
-                        const TopkScratch* scratch = nullptr);
+                        int32_t* sel, int32_t* sel_count, cudaStream_t st, const TopkScratch& scratch);
 cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, int64_t tok_end,
                                  const void* k, const KvPaging& pg, const float* fingerprints,
                                  const int32_t* unit_start,

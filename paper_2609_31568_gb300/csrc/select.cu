@@ -8,9 +8,9 @@
 //   k_stats   per (u, h): max_b z and 1 / sum_b exp(z - max) over the candidates
 //   k_vote    score[u][b] = sum_h exp(z[u][h][b] - max) / sum   (heads in order)
 //   k_topk    a radix select of the k-th largest key and an index-ordered
-//             compaction (up to 4096 candidates in shared memory; with a
-//             scratch area and more than 64K candidates, the multi-CTA form
-//             below): output ascending, ties to the lower b.
+//             compaction (up to 4096 candidates in shared memory; in the
+//             token-level selection with more than 64K candidates, the
+//             multi-CTA form below): output ascending, ties to the lower b.
 // Sequences of little selection work run in one kernel instead, k_select_few.
 //
 // Candidates of unit u are the blocks with a token in [n_sink, W_u),
@@ -1526,7 +1526,7 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
 }
 
 cudaError_t launch_topk(const Derived& d, const Units& ut, int sc_begin, int sc_end, const float* scores,
-                        int32_t* sel, int32_t* sel_count, cudaStream_t st, const TopkScratch* scratch)
+                        int32_t* sel, int32_t* sel_count, cudaStream_t st, const TopkScratch& scratch)
 {
     SelArgs a{};
     a.ut = ut;
@@ -1542,20 +1542,20 @@ cudaError_t launch_topk(const Derived& d, const Units& ut, int sc_begin, int sc_
     a.sigma = d.sigma;
     const int max_units = sc_end - sc_begin;
     if (max_units <= 0) return cudaSuccess;
-    if (!scratch || d.nb <= kMultiCtaMin) {
+    if (d.nb <= kMultiCtaMin) {
         k_topk<<<max_units, kTopkThreads, 0, st>>>(a, scores, sel, sel_count);
         return cudaGetLastError();
     }
     // many candidates per unit: chunks of kChunk keys over the whole GPU
-    auto* state = reinterpret_cast<TopkState*>(scratch->state);
-    const int mc = scratch->max_chunks;
+    auto* state = reinterpret_cast<TopkState*>(scratch.state);
+    const int mc = scratch.max_chunks;
     const dim3 grid(static_cast<unsigned>(mc), static_cast<unsigned>(max_units));
-    k_topk_init<<<max_units, 256, 0, st>>>(a, sel, sel_count, scratch->hist, state);
+    k_topk_init<<<max_units, 256, 0, st>>>(a, sel, sel_count, scratch.hist, state);
     for (int p = 0; p < kTopkPasses; ++p)
-        k_topk_hist<<<grid, kChunkThreads, 0, st>>>(a, scores, scratch->hist, state, p);
-    k_topk_count<<<grid, kChunkThreads, 0, st>>>(a, scores, scratch->hist, state, scratch->counts, mc);
-    k_topk_scan<<<max_units, 32, 0, st>>>(a, state, scratch->counts, mc, sel, sel_count);
-    k_topk_emit<<<grid, kChunkThreads, 0, st>>>(a, scores, state, scratch->counts, mc, sel);
+        k_topk_hist<<<grid, kChunkThreads, 0, st>>>(a, scores, scratch.hist, state, p);
+    k_topk_count<<<grid, kChunkThreads, 0, st>>>(a, scores, scratch.hist, state, scratch.counts, mc);
+    k_topk_scan<<<max_units, 32, 0, st>>>(a, state, scratch.counts, mc, sel, sel_count);
+    k_topk_emit<<<grid, kChunkThreads, 0, st>>>(a, scores, state, scratch.counts, mc, sel);
     return cudaGetLastError();
 }
 

@@ -905,7 +905,7 @@ cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, 
         const TopkScratch scratch{reinterpret_cast<int32_t*>(ws + lay.topk_hist),
                                   reinterpret_cast<int32_t*>(ws + lay.topk_state),
                                   reinterpret_cast<int2*>(ws + lay.topk_counts), topk_max_chunks(d)};
-        return launch_topk(d, a.ut, a.sc_begin, a.sc_end, a.scores, sel, sel_count, st, &scratch);
+        return launch_topk(d, a.ut, a.sc_begin, a.sc_end, a.scores, sel, sel_count, st, scratch);
     }
     const int tiles_u = (max_units + a.U - 1) / a.U;
     const dim3 grid(static_cast<unsigned>(a.n_ranges), static_cast<unsigned>(tiles_u));
@@ -925,7 +925,7 @@ cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, 
     const TopkScratch scratch{reinterpret_cast<int32_t*>(ws + lay.topk_hist),
                               reinterpret_cast<int32_t*>(ws + lay.topk_state),
                               reinterpret_cast<int2*>(ws + lay.topk_counts), topk_max_chunks(d)};
-    return launch_topk(d, a.ut, a.sc_begin, a.sc_end, a.scores, sel, sel_count, st, &scratch);
+    return launch_topk(d, a.ut, a.sc_begin, a.sc_end, a.scores, sel, sel_count, st, scratch);
 }
 
 }  // namespace scale
