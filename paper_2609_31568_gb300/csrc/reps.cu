@@ -52,10 +52,11 @@ struct StepArgs {
     int64_t m0;
     float* fp;
     float* ss_part;
-    // representatives of the blocks [b_base, ...): row_cols sixteen-byte columns
-    // of a key row per CTA, `splits` CTAs per block
-    int row_chunks, row_cols, groups, splits, B;
-    int64_t nb, b_base;
+    // representatives of the blocks [b_base, b_end): `per` blocks of `groups` row
+    // groups per CTA, row_cols sixteen-byte columns of a key row, `splits` CTAs
+    // per row
+    int row_chunks, row_cols, groups, per, splits, B;
+    int64_t nb, b_base, b_end;
     float* reps;
     // clusters
     int M, S_max, per_outer, c_begin, c_end;
@@ -67,47 +68,56 @@ struct StepArgs {
     int32_t* ticket;
 };
 
-// Representative key of one block for every KV head: the mean of the block's
-// keys. Thread c of row group g owns elements [8c, 8c + 8) of the token rows g,
-// g + groups, ... of the block (every row read as one coalesced span), with 8
-// loads in flight; the groups' sums are then added in group order, so the
-// result is bit-reproducible.
+// Representative keys of `per` neighbouring blocks for every KV head: the means
+// of the blocks' keys. Thread c of row group g of a block owns elements
+// [8c, 8c + 8) of the token rows g, g + groups, ... of the block (every row read
+// as one coalesced span), with 8 loads in flight; the groups' sums are then
+// added in group order, so the result is bit-reproducible. Few KV heads and
+// small blocks leave a block little to read: with 8 rows a group and as many
+// blocks as the CTA has threads for, step (a) over 160K tokens of one query and
+// one KV head takes 13.2 us in blocks of 64 (a block per CTA, 32 groups: 28.2 us).
+template <bool PAGED>
 __device__ void block_reps(const StepArgs& a, int item, float4* part)
 {
     const int c = threadIdx.x % a.row_cols;
-    const int g = threadIdx.x / a.row_cols;
-    const int64_t b = a.b_base + item / a.splits;
+    const int x = threadIdx.x / a.row_cols;
+    const int groups = a.groups, slot = x / groups, g = x - slot * groups;
+    const int64_t b = a.b_base + static_cast<int64_t>(item / a.splits) * a.per + slot;
     const int col = item % a.splits * a.row_cols + c;
-    const int groups = a.groups;
     const int64_t t0 = b * a.B;
     const int64_t t1 = (t0 + a.B < a.N) ? t0 + a.B : a.N;
-    const bool live = g < groups && col < a.row_chunks;
+    const bool live = slot < a.per && b < a.b_end && col < a.row_chunks;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (live) {
         const uint4* src = a.k + col;
         const uint4 zero = make_uint4(0, 0, 0, 0);
+        auto row = [&](int64_t t) {  // -1: a page outside the pool reads as zeros
+            const int64_t r = PAGED ? kv_row(a.pg, t) : t;
+            return PAGED && r < 0 ? zero : ld_stream(src + r * a.row_chunks);
+        };
         int64_t t = t0 + g;
         for (; t + 7 * groups < t1; t += 8 * groups) {
-            uint4 x[8];
+            uint4 v[8];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int64_t r = kv_row(a.pg, t + i * groups);  // -1: a page outside the pool reads as zeros
-                x[i] = r < 0 ? zero : ld_stream(src + r * a.row_chunks);
-            }
+            for (int i = 0; i < 8; ++i) v[i] = row(t + i * groups);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) add_bf16x8(acc, x[i]);
+            for (int i = 0; i < 8; ++i) add_bf16x8(acc, v[i]);
         }
-        for (; t < t1; t += groups) {
-            const int64_t r = kv_row(a.pg, t);
-            add_bf16x8(acc, r < 0 ? zero : ld_stream(src + r * a.row_chunks));
+        if (t < t1) {
+            uint4 v[7];
+#pragma unroll
+            for (int i = 0; i < 7; ++i) v[i] = t + i * groups < t1 ? row(t + i * groups) : zero;
+#pragma unroll
+            for (int i = 0; i < 7; ++i) add_bf16x8(acc, v[i]);
         }
-        part[(g * a.row_cols + c) * 2] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-        part[(g * a.row_cols + c) * 2 + 1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+        part[(x * a.row_cols + c) * 2] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        part[(x * a.row_cols + c) * 2 + 1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
     }
     __syncthreads();
     if (g != 0 || !live) return;
     for (int gg = 1; gg < groups; ++gg) {
-        const float4 lo = part[(gg * a.row_cols + c) * 2], hi = part[(gg * a.row_cols + c) * 2 + 1];
+        const int y = (x + gg) * a.row_cols + c;
+        const float4 lo = part[y * 2], hi = part[y * 2 + 1];
         acc[0] += lo.x; acc[1] += lo.y; acc[2] += lo.z; acc[3] += lo.w;
         acc[4] += hi.x; acc[5] += hi.y; acc[6] += hi.z; acc[7] += hi.w;
     }
@@ -148,7 +158,14 @@ __device__ void fingerprint(const StepArgs& a, int im, int cg, float4* red, floa
 #pragma unroll
             for (int u = 0; u < 8; ++u) add_bf16x8(acc, x[u]);
         }
-        for (; t < t1; t += kFpWarps) add_bf16x8(acc, ld_stream(src + t * D8));
+        if (t < t1) {
+            uint4 x[7];
+#pragma unroll
+            for (int u = 0; u < 7; ++u)
+                x[u] = t + u * kFpWarps < t1 ? ld_stream(src + (t + u * kFpWarps) * D8) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int u = 0; u < 7; ++u) add_bf16x8(acc, x[u]);
+        }
     }
     red[(w * kFpGroupCols + lane) * 2] = make_float4(acc[0], acc[1], acc[2], acc[3]);
     red[(w * kFpGroupCols + lane) * 2 + 1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
@@ -336,7 +353,8 @@ __global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __rest
 // query and 8 KV heads (1.35 GB) with a threshold take 199 us with k_gram,
 // 6.8 TB/s (222 us as four kernels); chunk by chunk with theta = -1 the eight
 // calls of that layer take 0.25 ms less, a 4K layer's one call 14 us less.
-__global__ void __launch_bounds__(kStepThreads, 2) k_step_a(const StepArgs a)
+template <bool PAGED, int CTAS>
+__global__ void __launch_bounds__(kStepThreads, CTAS) k_step_a(const StepArgs a)
 {
     __shared__ float4 part[kStepThreads * 2];
     __shared__ float wsum[8];
@@ -350,7 +368,7 @@ __global__ void __launch_bounds__(kStepThreads, 2) k_step_a(const StepArgs a)
     }
     --x;
     if (x < a.nm * a.fp_groups) fingerprint(a, x / a.fp_groups, x % a.fp_groups, part, wsum);
-    else block_reps(a, x - a.nm * a.fp_groups, part);
+    else block_reps<PAGED>(a, x - a.nm * a.fp_groups, part);
 }
 
 }  // namespace
@@ -397,11 +415,14 @@ cudaError_t launch_build_reps_range(const Derived& d, const void* q, const void*
     a.ss_part = ss_part;
     a.row_chunks = d.Hkv * (kHeadDim / 8);
     a.row_cols = a.row_chunks < kStepThreads ? a.row_chunks : kStepThreads;
-    a.groups = kStepThreads / a.row_cols;
+    const int slots = kStepThreads / a.row_cols;  // row groups of a CTA, eight rows or more each
+    a.groups = d.B / 8 < slots ? (d.B / 8 > 0 ? d.B / 8 : 1) : slots;
+    a.per = slots / a.groups;
     a.splits = (a.row_chunks + a.row_cols - 1) / a.row_cols;
     a.B = d.B;
     a.nb = d.nb;
     a.b_base = b0;
+    a.b_end = b1;
     a.reps = reps;
     a.M = static_cast<int>(d.M);
     a.S_max = d.S_max;
@@ -416,10 +437,19 @@ cudaError_t launch_build_reps_range(const Derived& d, const void* q, const void*
     a.ticket = reinterpret_cast<int32_t*>(ws + kTicketOffset);
 
     // block size 1 may skip the representatives: token-level selection reads K itself
-    const int64_t rep_ctas = reps && b1 > b0 ? (b1 - b0) * a.splits : 0;
+    const int64_t rep_ctas = reps && b1 > b0 ? (b1 - b0 + a.per - 1) / a.per * a.splits : 0;
     const int64_t grid = 1 + static_cast<int64_t>(a.nm) * a.fp_groups + rep_ctas;
     if (grid > 0x7FFFFFFFll) return cudaErrorInvalidConfiguration;
-    cudaError_t e = launch_after(st, dim3(static_cast<unsigned>(grid)), kStepThreads, 0, 1, k_step_a, a);
+    int sms = 0;
+    cudaError_t e = device_sms(&sms);
+    if (e != cudaSuccess) return e;
+    // Three CTAs per SM keep HBM busy while short sub-chunks are summed up, with 40
+    // registers instead of 64 for the loads in flight. 160K tokens of 28 heads on 4
+    // in sub-chunks of 128: 196 us (two per SM 228); of 2,048, 60K tokens of 32 on 8:
+    // 95.6 us (two per SM 88.7); even at 512.
+    const bool dense = d.L <= 512 && static_cast<int64_t>(a.nm) * a.fp_groups > 2ll * sms;
+    auto kern = pg.page_table ? k_step_a<true, 2> : dense ? k_step_a<false, 3> : k_step_a<false, 2>;
+    e = launch_after(st, dim3(static_cast<unsigned>(grid)), kStepThreads, 0, 1, kern, a);
     if (e == cudaSuccess && d.S_max > 1 && d.theta > -1.0f) {
         // a warp per cosine, and enough threads to compact the anchors
         const int warps = d.S_max - 1 < 8 ? 8 : d.S_max - 1 < 16 ? d.S_max - 1 : 16;
