@@ -39,8 +39,7 @@ __device__ __forceinline__ uint4 ld_stream(const uint4* p)
 constexpr int kFpWarps = 16;
 constexpr int kFpGroupCols = 32;  // sixteen-byte columns of a fingerprint CTA
 constexpr int kStepThreads = 32 * kFpWarps;
-constexpr int kBand = 4096;       // cosines that the clustering keeps in shared memory
-static_assert(kBand * sizeof(float) <= kStepThreads * 2 * sizeof(float4), "k_step_a's buffer");
+constexpr int kBand = 4096;       // cosines of a chunk that the clustering keeps in shared memory
 
 struct StepArgs {
     const uint4* q;
@@ -61,7 +60,7 @@ struct StepArgs {
     // clusters
     int M, S_max, per_outer, c_begin, c_end;
     float theta;
-    const float* gram;
+    float* gram;
     int32_t* flag;
     int32_t* unit_start;
     int32_t* n_units;
@@ -206,8 +205,8 @@ __device__ __forceinline__ float fp_norm(const float* __restrict__ ss_part, int 
     return sqrtf(s);
 }
 
-// Exclusive block scan of 0/1 flags; returns this thread's exclusive prefix,
-// *total receives the block total.
+// Exclusive block scan of the threads' counts; returns this thread's exclusive
+// prefix, *total receives the block total.
 __device__ int block_exclusive_scan(int f, int* sh, int* total)
 {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
@@ -234,78 +233,79 @@ __device__ int block_exclusive_scan(int f, int* sh, int* total)
     return excl;
 }
 
-// Algorithm 1 in the outer chunks [c_begin, c_end), by one CTA (one thread per
-// chunk walks its sub-chunks: the anchor a admits j while cos(v_a, v_j) >=
-// theta and |C_a| < S_max), which then compacts the anchor flags of those chunks
-// into unit_start, after the *n_units units of the chunks before c_begin.
-__device__ void cluster(const StepArgs& a, int* sh, float* band)
+// Algorithm 1 in outer chunk c: the anchor a admits j while cos(v_a, v_j) >= theta
+// and |C_a| < S_max. The walk is a chain of dependent cosines. By one thread, with
+// `band` the chunk's cosines in shared memory: 30 cycles a link instead of 700.
+__device__ void walk_band(const StepArgs& a, int c, const float* band)
 {
-    const int M = a.M, S_max = a.S_max, per_outer = a.per_outer, c_begin = a.c_begin, c_end = a.c_end;
-    const float theta = a.theta;
-    int32_t* flag = a.flag;
-    int32_t* unit_start = a.unit_start;
-    int32_t* n_units = a.n_units;
-    const bool always = theta <= -1.0f;
+    const int c0 = c * a.per_outer, c1 = min(a.M, c0 + a.per_outer);
+    for (int an = c0; an < c1;) {
+        a.flag[an] = 1;
+        int j = an + 1;
+        for (; j < c1 && j - an < a.S_max && band[(an - c0) * a.S_max + j - an] >= a.theta; ++j) a.flag[j] = 0;
+        an = j;
+    }
+}
+
+// By one warp, a lane per candidate of the anchor, with the cosines in memory:
+// one round of loads for a cluster of up to 33 sub-chunks.
+__device__ void walk_rows(const StepArgs& a, int c)
+{
+    const int lane = threadIdx.x & 31, c0 = c * a.per_outer, c1 = min(a.M, c0 + a.per_outer);
+    for (int an = c0; an < c1;) {
+        const int most = c1 - an < a.S_max ? c1 - an : a.S_max;
+        int size = 1;
+        for (int d0 = 1; d0 < most; d0 += 32) {
+            const int d = d0 + lane;
+            const float cs = d < most ? __ldcg(&a.gram[static_cast<int64_t>(an) * a.S_max + d]) : 0.f;
+            const unsigned out = __ballot_sync(0xFFFFFFFFu, d >= most || !(cs >= a.theta));
+            size = d0 + (out ? __ffs(out) - 1 : 32);
+            if (out) break;
+        }
+        for (int i = lane; i < size; i += 32) a.flag[an + i] = i == 0;
+        an += size;
+    }
+}
+
+// The anchors of the outer chunks [c_begin, c_end) into unit_start, after the
+// *n_units units of the chunks before c_begin, by one CTA: every thread a run of
+// sub-chunks, counted, and after one scan written. `full`: every cluster takes
+// S_max sub-chunks or what its outer chunk has left.
+__device__ void compact(const StepArgs& a, bool full, int* sh)
+{
+    const int M = a.M, m_begin = a.c_begin * a.per_outer, m_end = min(M, a.c_end * a.per_outer);
     // read before the first barrier; thread 0 rewrites it after the last
-    int offset = c_begin == 0 ? 0 : *n_units;
-    const int m_begin = c_begin * per_outer;
-    const int m_end = min(M, c_end * per_outer);
-    // cosine of sub-chunk an with sub-chunk j: cs(an, j - an)
-    auto walk = [&](int c, auto cs) {
-        const int c1 = min(M, (c + 1) * per_outer);
-        int an = c * per_outer;
-        while (an < c1) {
-            flag[an] = 1;
-            int size = 1, j = an + 1;
-            while (j < c1 && size < S_max) {
-                const bool admit = always || cs(an, j - an) >= theta;
-                if (!admit) break;
-                flag[j] = 0;
-                ++size;
-                ++j;
-            }
-            an = j;
-        }
-    };
-    // The walk is a chain of dependent cosines: their band is brought into shared
-    // memory, as many chunks at a time as fit (16 chunks of 16 sub-chunks: 30
-    // cycles a link instead of 700).
-    const int64_t per_chunk = static_cast<int64_t>(per_outer) * S_max;
-    if (!always && per_chunk <= kBand) {
-        const int batch = min(static_cast<int>(kBand / per_chunk), static_cast<int>(blockDim.x));
-        for (int cb = c_begin; cb < c_end; cb += batch) {
-            const int row0 = cb * per_outer;
-            const int rows = min(m_end, (cb + batch) * per_outer) - row0;
-            for (int i = threadIdx.x; i < rows * S_max; i += blockDim.x)
-                band[i] = __ldcg(&a.gram[static_cast<int64_t>(row0) * S_max + i]);
-            __syncthreads();
-            const int c = cb + static_cast<int>(threadIdx.x);
-            if (static_cast<int>(threadIdx.x) < batch && c < c_end)
-                walk(c, [&](int an, int d) { return band[(an - row0) * S_max + d]; });
-            __syncthreads();
-        }
-    } else {
-        for (int c = c_begin + static_cast<int>(threadIdx.x); c < c_end; c += blockDim.x)
-            walk(c, [&](int an, int d) { return __ldcg(&a.gram[static_cast<int64_t>(an) * S_max + d]); });
-    }
-    __syncthreads();
-    for (int base = m_begin; base < m_end; base += blockDim.x) {
-        const int i = base + threadIdx.x;
-        const int f = (i < m_end) ? flag[i] : 0;
-        int total;
-        const int excl = block_exclusive_scan(f, sh, &total);
-        if (f) unit_start[offset + excl] = i;
-        offset += total;
-    }
-    for (int i = offset + threadIdx.x; i <= M; i += blockDim.x) unit_start[i] = M;
-    if (threadIdx.x == 0) *n_units = offset;
+    const int offset = a.c_begin == 0 ? 0 : *a.n_units;
+    const int run = (m_end - m_begin + static_cast<int>(blockDim.x) - 1) / static_cast<int>(blockDim.x);
+    const int r0 = m_begin + static_cast<int>(threadIdx.x) * run, r1 = min(m_end, r0 + run);
+    auto is_anchor = [&](int i) { return full ? i % a.per_outer % a.S_max == 0 : __ldcg(&a.flag[i]) != 0; };
+    int count = 0, total;
+#pragma unroll 4
+    for (int i = r0; i < r1; ++i) count += is_anchor(i);
+    int at = offset + block_exclusive_scan(count, sh, &total);
+#pragma unroll 4
+    for (int i = r0; i < r1; ++i)
+        if (is_anchor(i)) a.unit_start[at++] = i;
+    for (int i = offset + total + static_cast<int>(threadIdx.x); i <= M; i += blockDim.x) a.unit_start[i] = M;
+    if (threadIdx.x == 0) *a.n_units = offset + total;
+}
+
+// Arrivals at the clusters of outer chunk c, counted in the unused cosine of its
+// first sub-chunk with itself.
+__device__ __forceinline__ int32_t* chunk_ticket(const StepArgs& a, float* gram, int c)
+{
+    return reinterpret_cast<int32_t*>(gram + static_cast<int64_t>(c) * a.per_outer * a.S_max);
 }
 
 // gram[i][d] = cos(v_i, v_{i+d}) = v~_i . v~_{i+d} for 1 <= d < S_max and i+d
 // in the same outer chunk; 0 when either norm is 0. One warp per (i, d);
-// one CTA per i in [m0, m0 + gridDim.x). The CTA that finishes last (a ticket
-// that k_step_a cleared) then forms the clusters of the range.
-__global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __restrict__ gram)
+// `rows` neighbouring i of one outer chunk per CTA. Where the cosines of all
+// chunks fit shared memory, the CTA that finishes last (a ticket that k_step_a
+// cleared) walks and compacts the clusters of all of them; else the last one of
+// every chunk walks the chunk and the last one of these compacts. Step (a) of 4K
+// tokens of one head in 32 sub-chunks: 12.5 us (19 with a ticket per chunk); of 1M
+// tokens in 8,192: 169 us (all chunks walked by the last CTA 608 us).
+__global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __restrict__ gram, int rows)
 {
     __shared__ int sh[40];
     __shared__ int last;
@@ -314,37 +314,63 @@ __global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __rest
     const float* fp = args.fp;
     const float* ss_part = args.ss_part;
     const int groups = args.fp_groups, D = args.D8 * 8, M = args.M, S_max = args.S_max, per_outer = args.per_outer;
-    const int i = static_cast<int>(args.m0) + static_cast<int>(blockIdx.x);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nw = blockDim.x >> 5;
-    const int chunk_end = min(M, (i / per_outer + 1) * per_outer);
-    for (int d = warp + 1; d < S_max; d += nw) {
-        const int j = i + d;
+    const int ctas = (per_outer + rows - 1) / rows;  // of a full chunk
+    const int c = args.c_begin + static_cast<int>(blockIdx.x) / ctas;
+    const int chunk = c * per_outer, chunk_end = min(M, chunk + per_outer);
+    const int i0 = chunk + static_cast<int>(blockIdx.x) % ctas * rows, i1 = min(chunk_end, i0 + rows);
+    for (int x = warp; x < (i1 - i0) * (S_max - 1); x += nw) {
+        const int i = i0 + (rows == 1 ? 0 : x / (S_max - 1)), d = x - (i - i0) * (S_max - 1) + 1, j = i + d;
         if (j >= chunk_end) continue;
         const float4* a = reinterpret_cast<const float4*>(fp + static_cast<int64_t>(i) * D);
         const float4* b = reinterpret_cast<const float4*>(fp + static_cast<int64_t>(j) * D);
         // 16-byte loads, four independent FMA chains (D is a multiple of 128)
         float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll 8
-        for (int c = lane; c < D / 4; c += 32) {
-            const float4 x = a[c], y = b[c];
-            s0 = fmaf(x.x, y.x, s0);
-            s1 = fmaf(x.y, y.y, s1);
-            s2 = fmaf(x.z, y.z, s2);
-            s3 = fmaf(x.w, y.w, s3);
+        for (int e = lane; e < D / 4; e += 32) {
+            const float4 u = a[e], v = b[e];
+            s0 = fmaf(u.x, v.x, s0);
+            s1 = fmaf(u.y, v.y, s1);
+            s2 = fmaf(u.z, v.z, s2);
+            s3 = fmaf(u.w, v.w, s3);
         }
         float s = (s0 + s1) + (s2 + s3);
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
         const float na = fp_norm(ss_part, groups, i), nb = fp_norm(ss_part, groups, j);  // whole warp
         if (lane == 0) gram[static_cast<int64_t>(i) * S_max + d] = (na > 0.f && nb > 0.f) ? s / (na * nb) : 0.f;
     }
-    __threadfence();
+    // whether this CTA is the last of `of` to get here
+    auto arrive = [&](int32_t* ticket, int of) {
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == of - 1;
+        __syncthreads();
+        __threadfence();
+        return last != 0;
+    };
+    const int chunks = args.c_end - args.c_begin;
+    const int64_t per_chunk = static_cast<int64_t>(per_outer) * S_max;
+    const int held = per_chunk * chunks <= kBand ? chunks : 1;  // chunks that a CTA walks
+    if (held == chunks) {
+        if (!arrive(args.ticket, static_cast<int>(gridDim.x))) return;
+    } else if (!arrive(chunk_ticket(args, gram, c), ctas)) {
+        return;
+    }
+    const int cw = held == chunks ? args.c_begin : c;
+    if (per_chunk <= kBand) {
+        const int row0 = cw * per_outer, n = (min(M, (cw + held) * per_outer) - row0) * S_max;
+#pragma unroll 4
+        for (int x = threadIdx.x; x < n; x += blockDim.x) band[x] = __ldcg(gram + static_cast<int64_t>(row0) * S_max + x);
+        __syncthreads();
+        for (int x = threadIdx.x; x < held; x += blockDim.x) walk_band(args, cw + x, band + x * per_chunk);
+        __syncthreads();
+    } else if (warp == 0) {
+        walk_rows(args, cw);
+    }
+    if (held < chunks && !arrive(args.ticket, chunks)) return;
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(args.ticket, 1) == static_cast<int>(gridDim.x) - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    cluster(args, sh, band);
+    compact(args, false, sh);
 }
 
 // Roles by CTA: the clusters where they need no cosine (one CTA), then the
@@ -362,8 +388,13 @@ __global__ void __launch_bounds__(kStepThreads, CTAS) k_step_a(const StepArgs a)
     scale_ptx::pdl_enter();
     int x = blockIdx.x;
     if (x == 0) {
-        if (threadIdx.x == 0) *a.ticket = 0;
-        if (a.theta <= -1.0f || a.S_max == 1) cluster(a, sh, reinterpret_cast<float*>(part));
+        if (a.theta <= -1.0f || a.S_max == 1) {
+            compact(a, true, sh);
+        } else {
+            if (threadIdx.x == 0) *a.ticket = 0;
+            for (int c = a.c_begin + static_cast<int>(threadIdx.x); c < a.c_end; c += kStepThreads)
+                *chunk_ticket(a, a.gram, c) = 0;
+        }
         return;
     }
     --x;
@@ -451,9 +482,13 @@ cudaError_t launch_build_reps_range(const Derived& d, const void* q, const void*
     auto kern = pg.page_table ? k_step_a<true, 2> : dense ? k_step_a<false, 3> : k_step_a<false, 2>;
     e = launch_after(st, dim3(static_cast<unsigned>(grid)), kStepThreads, 0, 1, kern, a);
     if (e == cudaSuccess && d.S_max > 1 && d.theta > -1.0f) {
-        // a warp per cosine, and enough threads to compact the anchors
+        // Several sub-chunks per CTA where there are many more than SMs for them;
+        // a warp per cosine, and enough threads to compact the anchors.
+        const int many = a.nm / (2 * sms);
+        const int rows = many < 1 ? 1 : many < d.per_outer ? many : d.per_outer;
+        const int64_t ctas = static_cast<int64_t>(c_end - c_begin) * ((d.per_outer + rows - 1) / rows);
         const int warps = d.S_max - 1 < 8 ? 8 : d.S_max - 1 < 16 ? d.S_max - 1 : 16;
-        e = launch_after(st, dim3(static_cast<unsigned>(a.nm)), 32 * warps, 0, 1, k_gram, a, gram);
+        e = launch_after(st, dim3(static_cast<unsigned>(ctas)), 32 * warps, 0, 1, k_gram, a, gram, rows);
     }
     return e;
 }
