@@ -14,6 +14,8 @@
 // against 2,048 bytes per token and unit for 32 query heads on 8 KV heads.
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "launch.cuh"
 #include "ptx_sm103.cuh"
 #include "scale_internal.h"
@@ -36,6 +38,7 @@ constexpr int kLgFold = 16;                     // key tiles summed before they 
 constexpr int kLgCols = 16;                     // (unit, head) columns of a tile
 constexpr uint32_t kLgTile = 128 * 128 * 2;     // 128 keys x 128 dims, two 64-dim halves
 constexpr uint32_t kLgHalf = kLgTile / 2;
+constexpr float kFar = 1073741824.0f;           // 2^30: references whose neighbours are 64 apart
 constexpr uint32_t kLgOpMax = 3 * kLgCols * 256;  // query operand: up to 48 rows of 256 bytes
 constexpr uint32_t kLgSmem = kLgOpMax + kLgStages * kLgTile + 1024;
 static_assert(kLgOpMax % 1024 == 0, "key stages must stay 1024-aligned");
@@ -377,28 +380,61 @@ k_key_logits(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUt
                 }
                 tc_fence_before();
                 mbar_arrive(&bars.d_empty[b]);
-                const int t = lo + 128 * tile + r;
+                const int t0 = lo + 128 * tile, t = t0 + r;
                 float* zt = a.z + (static_cast<int64_t>(ui0) * a.Hq + j * G) * a.z_stride + t;
+                // The reference m is a whole number, so that every factor between
+                // references is an exact power of two, and z scale2 - m is rounded
+                // once, by the size of the difference. (With the product rounded
+                // first and references raised by jumps of 2^8, the scores of logits of
+                // standard deviation 3 were 31e-8 from 64 bits at 100,003 tokens; now
+                // 10e-8.) Beyond kFar the rounding of the product alone is larger than
+                // the exponential's range: a thread's sum then counts as 1, at the end.
+                // The raise stays as short as this: one instruction more, and the
+                // compiler no longer predicates it, which costs 12 %.
+                auto raise = [&](int c, float& x) {
+                    const float top = ceilf(z[c] * a.scale2), f = ex2(m[c] - top);
+                    sm[c] *= f;
+                    tot[c] *= f;
+                    m[c] = top;
+                    x = fminf(fmaf(z[c], a.scale2, -top), 1.0f);
+                };
+                // A tile of candidates of every unit (the windows ascend) goes through
+                // its units without a test per value, and looks for a larger reference
+                // once: 8 units at 300K tokens, 28 heads on 4, 222 us (a test per value
+                // 260), one unit at 1M, 32 on 8, 375 us (386).
+                if (t0 >= a.n_sink && t0 + 127 < s_W[0]) {
+                    float x[US * G], most = -INFINITY;
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const int ul = c / G, hl = c % G;
-                    if (ul < n_u && t >= a.n_sink && t < s_W[ul < US ? ul : 0]) {
-                        zt[(static_cast<int64_t>(ul) * a.Hq + hl) * a.z_stride] = z[c];
-                        // The reference m is a whole number, so that every factor
-                        // between references is an exact power of two, and z scale2 -
-                        // m is rounded once, by the size of the difference. (With the
-                        // product rounded first and references raised by jumps of 2^8,
-                        // the scores of logits of standard deviation 3 were 31e-8 from
-                        // 64 bits at 100,003 tokens; now 10e-8.)
-                        float x = fmaf(z[c], a.scale2, -m[c]);
-                        if (x > 0.0f) {
-                            const float top = ceilf(z[c] * a.scale2), f = ex2(m[c] - top);
-                            sm[c] *= f;
-                            tot[c] *= f;
-                            m[c] = top;
-                            x = fmaf(z[c], a.scale2, -top);
+                    for (int ul = 0; ul < US; ++ul) {
+                        if (ul >= n_u) break;
+#pragma unroll
+                        for (int c = ul * G; c < (ul + 1) * G && c < NC; ++c) {
+                            zt[(static_cast<int64_t>(ul) * a.Hq + c % G) * a.z_stride] = z[c];
+                            x[c] = fmaf(z[c], a.scale2, -m[c]);
+                            most = fmaxf(most, x[c]);
                         }
-                        sm[c] += ex2(x);
+                    }
+                    if (most > 0.0f) {
+#pragma unroll
+                        for (int c = 0; c < US * G && c < NC; ++c)
+                            if (c / G < n_u && x[c] > 0.0f) raise(c, x[c]);
+                    }
+#pragma unroll
+                    for (int ul = 0; ul < US; ++ul) {
+                        if (ul >= n_u) break;
+#pragma unroll
+                        for (int c = ul * G; c < (ul + 1) * G && c < NC; ++c) sm[c] += ex2(x[c]);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < NC; ++c) {
+                        const int ul = c / G, hl = c % G;
+                        if (ul < n_u && t >= a.n_sink && t < s_W[ul < US ? ul : 0]) {
+                            zt[(static_cast<int64_t>(ul) * a.Hq + hl) * a.z_stride] = z[c];
+                            float x = fmaf(z[c], a.scale2, -m[c]);
+                            if (x > 0.0f) raise(c, x);
+                            sm[c] += ex2(x);
+                        }
                     }
                 }
                 if (++fresh == kLgFold) {
@@ -417,6 +453,7 @@ k_key_logits(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUt
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
                     tot[c] += sm[c];
+                    if (fabsf(m[c]) >= kFar && m[c] > -INFINITY) tot[c] = 1.0f;
                     sm[c] = m[c];  // from here on this thread's own reference
                     for (int o = 16; o > 0; o >>= 1) m[c] = fmaxf(m[c], __shfl_xor_sync(0xFFFFFFFFu, m[c], o));
                     if (lane == 0) s_max[q][c] = m[c];
@@ -591,50 +628,57 @@ __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
         for (int i = tid; i < kVtCopies * kVoteBins; i += kVtThreads) (&s_hist[0][0])[i] = 0;
         __syncthreads();
         // the vote: four tokens per thread, the loads of kVoteGroup planes in
-        // flight, added as a tree, the groups in order
-        for (int i = 4 * tid; i < v1; i += 4 * kVtThreads) {
-            const float* zt = z + c0 + i;
-            float sc[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int h0 = 0; h0 < a.Hq; h0 += kVoteGroup) {
-                float4 x[kVoteGroup];
+        // flight, added as a tree, the groups in order; `far`: with the product
+        // rounded first, as the reference's was, so that its token keeps its weight
+        auto vote = [&](auto far) {
+            for (int i = 4 * tid; i < v1; i += 4 * kVtThreads) {
+                const float* zt = z + c0 + i;
+                float sc[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int h0 = 0; h0 < a.Hq; h0 += kVoteGroup) {
+                    float4 x[kVoteGroup];
 #pragma unroll
-                for (int e = 0; e < kVoteGroup; ++e)
-                    if (h0 + e < a.Hq)
-                        x[e] = __ldcg(reinterpret_cast<const float4*>(zt + static_cast<int64_t>(h0 + e) * a.z_stride));
+                    for (int e = 0; e < kVoteGroup; ++e)
+                        if (h0 + e < a.Hq)
+                            x[e] = __ldcg(reinterpret_cast<const float4*>(zt + static_cast<int64_t>(h0 + e) * a.z_stride));
 #pragma unroll
-                for (int e = 0; e < kVoteGroup; ++e) {
-                    const float2 st = h0 + e < a.Hq ? s_stat[h0 + e] : make_float2(INFINITY, 0.f);
-                    if (h0 + e >= a.Hq) x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    x[e].x = ex2(fmaf(x[e].x, a.scale2, -st.x)) * st.y;
-                    x[e].y = ex2(fmaf(x[e].y, a.scale2, -st.x)) * st.y;
-                    x[e].z = ex2(fmaf(x[e].z, a.scale2, -st.x)) * st.y;
-                    x[e].w = ex2(fmaf(x[e].w, a.scale2, -st.x)) * st.y;
-                }
-#pragma unroll
-                for (int w = kVoteGroup / 2; w > 0; w >>= 1)
-#pragma unroll
-                    for (int e = 0; e < w; ++e) {
-                        x[e].x += x[e + w].x;
-                        x[e].y += x[e + w].y;
-                        x[e].z += x[e + w].z;
-                        x[e].w += x[e + w].w;
+                    for (int e = 0; e < kVoteGroup; ++e) {
+                        const float2 st = h0 + e < a.Hq ? s_stat[h0 + e] : make_float2(INFINITY, 0.f);
+                        if (h0 + e >= a.Hq) x[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        auto weight = [&](float v) {
+                            return ex2(decltype(far)::value ? __fmul_rn(v, a.scale2) - st.x : fmaf(v, a.scale2, -st.x)) * st.y;
+                        };
+                        x[e] = make_float4(weight(x[e].x), weight(x[e].y), weight(x[e].z), weight(x[e].w));
                     }
-                sc[0] += x[0].x;
-                sc[1] += x[0].y;
-                sc[2] += x[0].z;
-                sc[3] += x[0].w;
-            }
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (i + e < v0 || i + e >= v1) continue;
-                if (scores) scores[c0 + i + e] = sc[e];
-                if (rank) {
-                    const uint32_t key = float_key(sc[e]);
-                    keys[i + e] = key;
-                    atomicAdd(&s_hist[warp % kVtCopies][key >> 21], 1);
+                    for (int w = kVoteGroup / 2; w > 0; w >>= 1)
+#pragma unroll
+                        for (int e = 0; e < w; ++e) {
+                            x[e].x += x[e + w].x;
+                            x[e].y += x[e + w].y;
+                            x[e].z += x[e + w].z;
+                            x[e].w += x[e + w].w;
+                        }
+                    sc[0] += x[0].x;
+                    sc[1] += x[0].y;
+                    sc[2] += x[0].z;
+                    sc[3] += x[0].w;
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (i + e < v0 || i + e >= v1) continue;
+                    if (scores) scores[c0 + i + e] = sc[e];
+                    if (rank) {
+                        const uint32_t key = float_key(sc[e]);
+                        keys[i + e] = key;
+                        atomicAdd(&s_hist[warp % kVtCopies][key >> 21], 1);
+                    }
                 }
             }
-        }
+        };
+        int far = 0;
+        for (int h = tid; h < a.Hq; h += kVtThreads) far |= fabsf(s_stat[h].x) >= kFar;
+        if (__syncthreads_or(far)) vote(std::true_type{});
+        else vote(std::false_type{});
         if (!rank) continue;
 
         uint32_t prefix = 0;

@@ -141,6 +141,29 @@ def test_error_of_spread_logits(n, spread):
     assert mean < 1.6e-7, mean
 
 
+@pytest.mark.parametrize("scale", [1e3, 1e9, 1e15, 1e30])
+def test_one_token_far_above_the_others(scale):
+    """A logit whose own rounding is larger than the range of the exponential: its token has the whole
+    probability of every head, in a tile of candidates and in the last, partial one."""
+    n, sub, topk = 3000, 1000, 300
+    assert _planes_fit(4, 1, n, sub, 0, topk)
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    keys = torch.randn(n, 1, 128, generator=gen, device="cuda", dtype=torch.bfloat16)
+    keys[:, 0, 0] = 0.0
+    keys[700, 0, 0], keys[1990, 0, 0] = scale, -scale
+    fp = 0.1 * torch.randn(3, 4, 128, generator=gen, device="cuda")
+    fp[:, :, 0] = 0.77
+    p = S.params(num_q_heads=4, num_kv_heads=1, sub_chunk=sub, n_tokens=n, max_cluster_subchunks=1, block_size=1,
+                 top_k=topk, n_sink=0, n_local=0)
+    buf = pkg.allocate(p, PER_SUB, want_scores=True)
+    S.scale_select_tokens(p, PER_SUB, 0, n, keys, fp.flatten(1), None, None, buf.sel_blocks, buf.sel_count,
+                          buf.sel_scores, buf.ws)
+    for u in (1, 2):
+        scores = buf.sel_scores[u, : u * sub]
+        assert torch.all(torch.isfinite(scores)) and 3.99 < float(scores[700]) < 4.01
+        assert float(scores.sum() - scores[700]) < 1e-3 and 700 in buf.sel_blocks[u].tolist()
+
+
 def _near(got, want, ref, sink, rel):
     """Whether every token in only one of the lists scores within `rel` of the k-th score."""
     kth = ref[want - sink].min()
