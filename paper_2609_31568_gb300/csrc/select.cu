@@ -54,6 +54,7 @@ struct SelArgs {
     int64_t nb;
     int B, k, n_sink, n_local;
     float sigma;
+    int scored;           // scores are asked for: also of units that take every candidate
     int32_t* status;      // device status word (bounded waits of k_logits)
     uint64_t timeout_ns;
 };
@@ -160,7 +161,7 @@ __global__ void __launch_bounds__(kLtThreads, 1) k_logits(SelArgs a, int seg, co
     int anc;
     unit_range(a.ut, u0 + n_u - 1, &anc, &s, &e);
     cand_range(a, s, &lo, &hi);
-    if (hi <= b0 || lo >= b0 + 128 || lo >= hi) return;
+    if (hi <= b0 || lo >= b0 + 128 || lo >= hi || (!a.scored && hi - lo <= a.k)) return;
     for (int i = tid; i < n_u; i += kLtThreads) {
         unit_range(a.ut, u0 + i, &anc, &s, &e);
         cand_range(a, s, &lo, &hi);
@@ -1482,6 +1483,7 @@ cudaError_t launch_select(const Derived& d, int mode, int64_t tok_begin, int64_t
     a.n_sink = d.n_sink;
     a.n_local = d.n_local;
     a.sigma = d.sigma;
+    a.scored = sel_scores != nullptr;
     a.status = reinterpret_cast<int32_t*>(ws + kStatusOffset);
     a.timeout_ns = timeout_ns;
     const int max_units = a.sc_end - a.sc_begin;  // units in range <= sub-chunks in range
