@@ -342,8 +342,7 @@ struct DecWs {
     size_t zpart;    // float2 [H_q][n_stat]               partial softmax sums of the logits
     size_t o_part;   // float4 [H_q][kDecMaxSplits][32]    attention: unnormalised outputs
     size_t ml_part;  // float2 [H_q][kDecMaxSplits]        (max, sum)
-    size_t tickets;  // int32 [H_kv]
-    size_t gate;     // int32 [1]
+    size_t tickets;  // int32 [H_kv], then the gate
     size_t scratch;  // int32 [kVoteScratchInts]           vote and top-k
     size_t end;
     int64_t z_stride, n_stat;
@@ -365,8 +364,7 @@ DecWs decode_layout(const Derived& d)
     w.zpart = take(heads * w.n_stat * sizeof(float2));
     w.o_part = take(heads * kDecMaxSplits * kHeadDim * sizeof(float));
     w.ml_part = take(heads * kDecMaxSplits * sizeof(float2));
-    w.tickets = take(static_cast<size_t>(d.Hkv) * sizeof(int32_t));
-    w.gate = take(sizeof(int32_t));
+    w.tickets = take((static_cast<size_t>(d.Hkv) + 1) * sizeof(int32_t));
     w.scratch = take(kVoteScratchInts * sizeof(int32_t));
     w.end = off;
     return w;
@@ -408,7 +406,7 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     const DecWs lay = decode_layout(d);
     auto* z = reinterpret_cast<float*>(ws + lay.z);
     auto* zpart = reinterpret_cast<float2*>(ws + lay.zpart);
-    auto* gate = reinterpret_cast<int32_t*>(ws + lay.gate);
+    auto* gate = reinterpret_cast<int32_t*>(ws + lay.tickets) + d.Hkv;
     auto* scratch = reinterpret_cast<int32_t*>(ws + lay.scratch);
 
     DecArgs a;
