@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
     __shared__ int s_hist[kVtCopies][kVoteBins];
     __shared__ float2 s_stat[kVtMaxHeads];
     __shared__ int s_scan[kVtWarps], s_gt[kVtWarps], s_eq[kVtWarps];
-    __shared__ int s_digit, s_need;
+    __shared__ int s_digit, s_need, s_far;
     pdl_trigger();  // launched plainly: what is before it has completed
     if (a.gate && !*a.gate) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -613,6 +613,7 @@ __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
             if (!scores || n == 0) continue;
         }
         // statistics: one warp per head; the parts in a fixed interleave and tree
+        if (tid == 0) s_far = 0;
         __syncthreads();
         for (int h = warp; h < a.Hq; h += kVtWarps) {
             const float2* pr = a.part + (static_cast<int64_t>(ui) * a.Hq + h) * a.n_part;
@@ -623,7 +624,10 @@ __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
             for (int x = x0; x < x1; x += 32)
                 if (pr[x].x > -INFINITY) s += pr[x].y * ex2(pr[x].x - m);
             for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
-            if (lane == 0) s_stat[h] = make_float2(m, s > 0.f ? 1.0f / s : 0.f);
+            if (lane == 0) {
+                s_stat[h] = make_float2(m, s > 0.f ? 1.0f / s : 0.f);
+                if (fabsf(m) >= kFar) s_far = 1;
+            }
         }
         for (int i = tid; i < kVtCopies * kVoteBins; i += kVtThreads) (&s_hist[0][0])[i] = 0;
         __syncthreads();
@@ -675,9 +679,7 @@ __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
                 }
             }
         };
-        int far = 0;
-        for (int h = tid; h < a.Hq; h += kVtThreads) far |= fabsf(s_stat[h].x) >= kFar;
-        if (__syncthreads_or(far)) vote(std::true_type{});
+        if (s_far) vote(std::true_type{});
         else vote(std::false_type{});
         if (!rank) continue;
 
