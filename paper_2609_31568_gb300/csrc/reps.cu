@@ -137,7 +137,8 @@ __device__ void block_reps(const StepArgs& a, int item, float4* part)
 // |X_i| and written, together with the group's sum of squares (the norm of
 // Sec. V-A1 adds those in group order). The order is fixed, so the result is
 // bit-reproducible and the same for a sub-chunk whichever range of sub-chunks
-// a launch covers.
+// a launch covers. IN: loads in flight of a thread.
+template <int IN>
 __device__ void fingerprint(const StepArgs& a, int im, int cg, float4* red, float* wsum)
 {
     const int64_t i = a.m0 + im;
@@ -150,20 +151,20 @@ __device__ void fingerprint(const StepArgs& a, int im, int cg, float4* red, floa
     if (c < D8) {
         const uint4* src = a.q + c;
         int64_t t = t0 + w;
-        for (; t + 7 * kFpWarps < t1; t += 8 * kFpWarps) {
-            uint4 x[8];
+        for (; t + (IN - 1) * kFpWarps < t1; t += IN * kFpWarps) {
+            uint4 x[IN];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = ld_stream(src + (t + u * kFpWarps) * D8);
+            for (int u = 0; u < IN; ++u) x[u] = ld_stream(src + (t + u * kFpWarps) * D8);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) add_bf16x8(acc, x[u]);
+            for (int u = 0; u < IN; ++u) add_bf16x8(acc, x[u]);
         }
         if (t < t1) {
-            uint4 x[7];
+            uint4 x[IN - 1];
 #pragma unroll
-            for (int u = 0; u < 7; ++u)
+            for (int u = 0; u < IN - 1; ++u)
                 x[u] = t + u * kFpWarps < t1 ? ld_stream(src + (t + u * kFpWarps) * D8) : make_uint4(0, 0, 0, 0);
 #pragma unroll
-            for (int u = 0; u < 7; ++u) add_bf16x8(acc, x[u]);
+            for (int u = 0; u < IN - 1; ++u) add_bf16x8(acc, x[u]);
         }
     }
     red[(w * kFpGroupCols + lane) * 2] = make_float4(acc[0], acc[1], acc[2], acc[3]);
@@ -247,8 +248,36 @@ __device__ void walk_band(const StepArgs& a, int c, const float* band)
     }
 }
 
+// By the CTA, with the cosines of as many sub-chunks at a time as shared memory
+// holds: step (a) of 512K tokens of 4 heads on one, an outer chunk of 4,096
+// sub-chunks and each a cluster, takes 552 us (a load per link: 1,543).
+__device__ void walk_windows(const StepArgs& a, int c, float* band, int* next)
+{
+    const int c1 = min(a.M, (c + 1) * a.per_outer), S_max = a.S_max;
+    for (int an = c * a.per_outer; an < c1;) {
+        const int rows = min(c1 - an, kBand / S_max);
+        const float* src = a.gram + static_cast<int64_t>(an) * S_max;
+#pragma unroll 4
+        for (int x = threadIdx.x; x < rows * S_max; x += blockDim.x) band[x] = __ldcg(src + x);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int at = an;
+            while (at < an + rows) {
+                a.flag[at] = 1;
+                int j = at + 1;
+                for (; j < c1 && j - at < S_max && band[(at - an) * S_max + j - at] >= a.theta; ++j) a.flag[j] = 0;
+                at = j;
+            }
+            *next = at;
+        }
+        __syncthreads();
+        an = *next;
+        __syncthreads();
+    }
+}
+
 // By one warp, a lane per candidate of the anchor, with the cosines in memory:
-// one round of loads for a cluster of up to 33 sub-chunks.
+// clusters that may be longer than shared memory.
 __device__ void walk_rows(const StepArgs& a, int c)
 {
     const int lane = threadIdx.x & 31, c0 = c * a.per_outer, c1 = min(a.M, c0 + a.per_outer);
@@ -280,12 +309,16 @@ __device__ void compact(const StepArgs& a, bool full, int* sh)
     const int r0 = m_begin + static_cast<int>(threadIdx.x) * run, r1 = min(m_end, r0 + run);
     auto is_anchor = [&](int i) { return full ? i % a.per_outer % a.S_max == 0 : __ldcg(&a.flag[i]) != 0; };
     int count = 0, total;
+    uint32_t first = 0;  // the run's first 32 are read once
 #pragma unroll 4
-    for (int i = r0; i < r1; ++i) count += is_anchor(i);
+    for (int i = r0; i < r1; ++i) {
+        const uint32_t f = is_anchor(i);
+        count += f;
+        if (i - r0 < 32) first |= f << (i - r0);
+    }
     int at = offset + block_exclusive_scan(count, sh, &total);
-#pragma unroll 4
     for (int i = r0; i < r1; ++i)
-        if (is_anchor(i)) a.unit_start[at++] = i;
+        if (i - r0 < 32 ? first >> (i - r0) & 1u : is_anchor(i)) a.unit_start[at++] = i;
     for (int i = offset + total + static_cast<int>(threadIdx.x); i <= M; i += blockDim.x) a.unit_start[i] = M;
     if (threadIdx.x == 0) *a.n_units = offset + total;
 }
@@ -365,6 +398,8 @@ __global__ void __launch_bounds__(512) k_gram(const StepArgs args, float* __rest
         __syncthreads();
         for (int x = threadIdx.x; x < held; x += blockDim.x) walk_band(args, cw + x, band + x * per_chunk);
         __syncthreads();
+    } else if (S_max <= kBand) {
+        walk_windows(args, cw, band, &last);
     } else if (warp == 0) {
         walk_rows(args, cw);
     }
@@ -398,7 +433,7 @@ __global__ void __launch_bounds__(kStepThreads, CTAS) k_step_a(const StepArgs a)
         return;
     }
     --x;
-    if (x < a.nm * a.fp_groups) fingerprint(a, x / a.fp_groups, x % a.fp_groups, part, wsum);
+    if (x < a.nm * a.fp_groups) fingerprint<CTAS == 1 ? 16 : 8>(a, x / a.fp_groups, x % a.fp_groups, part, wsum);
     else block_reps<PAGED>(a, x - a.nm * a.fp_groups, part);
 }
 
@@ -477,9 +512,13 @@ cudaError_t launch_build_reps_range(const Derived& d, const void* q, const void*
     // Three CTAs per SM keep HBM busy while short sub-chunks are summed up, with 40
     // registers instead of 64 for the loads in flight. 160K tokens of 28 heads on 4
     // in sub-chunks of 128: 196 us (two per SM 228); of 2,048, 60K tokens of 32 on 8:
-    // 95.6 us (two per SM 88.7); even at 512.
-    const bool dense = d.L <= 512 && static_cast<int64_t>(a.nm) * a.fp_groups > 2ll * sms;
-    auto kern = pg.page_table ? k_step_a<true, 2> : dense ? k_step_a<false, 3> : k_step_a<false, 2>;
+    // 95.6 us (two per SM 88.7); even at 512. Where a second CTA per SM has little to
+    // do a CTA's own loads decide: 16 in flight instead of 8 (3K tokens of 16 heads
+    // on 8 in sub-chunks of 2,048).
+    const int64_t fps = static_cast<int64_t>(a.nm) * a.fp_groups;
+    auto kern = pg.page_table ? k_step_a<true, 2>
+                : grid <= sms ? k_step_a<false, 1>
+                : d.L <= 512 && d.B <= 512 && fps > 2ll * sms ? k_step_a<false, 3> : k_step_a<false, 2>;
     e = launch_after(st, dim3(static_cast<unsigned>(grid)), kStepThreads, 0, 1, kern, a);
     if (e == cudaSuccess && d.S_max > 1 && d.theta > -1.0f) {
         // Several sub-chunks per CTA where there are many more than SMs for them;

@@ -40,7 +40,8 @@ def _clusters(topic, per_outer, cap):
     (5, 4, 2, 0.5),
     (300, 16, 16, 0.9),
     (2000, 40, 40, 0.99),    # a cluster takes two rounds of a warp
-    (700, 600, 9, 0.8),      # 5,400 cosines of a chunk
+    (700, 600, 9, 0.8),      # 5,400 cosines of a chunk: two windows of 455 sub-chunks
+    (900, 900, 5000, 0.9),   # an anchor's cosines do not fit shared memory
     (130, 64, 64, 0.97),     # 4,096: the most that shared memory keeps
     (8200, 8, 8, 0.7),       # 1,025 chunks
     (3000, 3, 2, 0.0),       # every sub-chunk a cluster
