@@ -94,7 +94,7 @@ __host__ __device__ __forceinline__ int64_t window_start(int n_local, int64_t t)
 // order in shared memory; the CTA that finishes last for a KV head (a ticket
 // counter) merges the splits of its heads in order and writes the bf16 output.
 // Bound by latency and issue: 38 MB of K and V at k = 8192 (5.6 us of HBM time)
-// take 14.6 us from L2 (before: a warp per head and a combine kernel, 44 us).
+// take 17 us alone with cold caches (before: a warp per head and a combine kernel, 44 us).
 // Also stores what the step's reuse decision changes: the state words and, when
 // the step retrieved, the anchor.
 template <int G>
@@ -489,7 +489,8 @@ cudaError_t launch_decode_step(const Derived& d, int64_t t, const void* q, const
     }
     if (e != cudaSuccess) return e;
 
-    // Splits: one CTA per SM, and at least 64 keys each.
+    // Splits: at most one CTA per SM (one and two KV heads: kDecMaxSplits each), and
+    // at least 64 keys each.
     int sms = 0;
     if ((e = device_sms(&sms)) != cudaSuccess) return e;
     const int64_t n_max = d.n_sink + static_cast<int64_t>(d.k) + (t - W + 1);

@@ -145,10 +145,10 @@ __device__ bool decode_retrieves(const KeyScoreArgs& a)
 // (max, sum) in the token's thread, merged over the 128 threads (a butterfly,
 // then the four warps in order) when the head changes. Bound by reading K,
 // with many unit tiles by the planes. The CTAs of the unit tiles that read the
-// same keys run side by side when L2 does not hold all keys: 16 units of 32
-// heads take 114.8 us at 48K tokens, 218.5 at 128K and 974 at 512K (tile after
-// tile 122.3, 241.7 and 1098); when it does that only loses (40K tokens: 100
-// against 98.2).
+// same keys run side by side when L2 does not hold all keys: selection calls of
+// 16 units of 32 heads take 107 us at 48K tokens, 208 at 128K and 896 at 512K
+// (tile after tile 121, 256 and 1018); where L2 holds them the order matters
+// little (40K tokens: 98.2 side by side, 100.6 tile after tile, which is taken).
 template <int G, int PARTS>
 __global__ void __launch_bounds__(kLgThreads, 2)
 k_key_logits(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUtensorMap tk, const KeyScoreArgs a)
@@ -248,10 +248,10 @@ k_key_logits(const __grid_constant__ CUtensorMap tf, const __grid_constant__ CUt
             tma_prefetch_desc(&tk);
             // Keys beyond what L2 holds leave it before the planes that the vote
             // reads, as long as L2 holds those: a decode step of 32 heads takes
-            // 87.3 us at 128K tokens and 221.9 at 512K (a plane of 64 MB), 94.5
-            // and 227.3 without. Planes larger than L2 are read from HBM all the
-            // same, and the policy only costs: 411.7 us at 1M, 407 without; 16
-            // units at 256K tokens 508 and 493.
+            // 84.7 us at 128K tokens and 223.2 at 512K (a plane of 64 MB), 92.1
+            // and 229.3 without. Planes larger than L2 are read from HBM all the
+            // same, and the policy only costs: 416.9 us at 1M, 412.5 without; a
+            // selection of 16 units at 256K tokens 477 and 381.
             const int64_t plane = items * 128 * G * 4 * (u_end - u_first);
             const bool stream = items * static_cast<int64_t>(kLgTile) > kLgStreamBytes && plane <= kLgPlaneBytes;
             const uint64_t policy = policy_evict_first();
@@ -561,8 +561,8 @@ __device__ bool group_barrier(int32_t* counter, int target, uint64_t timeout_ns,
 // T and the first `need` equal to it; the CTAs' counts are exchanged at the
 // last barrier, and each CTA writes its picks in token order. Bound by reading
 // the plane and, below some 100K tokens, by its four barriers of about 2 us.
-// Measured for one unit with 32 heads: 52 us at 1M tokens (20 us of HBM time)
-// and 26 us at 128K, against 142 and about 60 us for the statistics, the vote
+// Measured for one unit with 32 heads: 50 us at 1M tokens (20 us of HBM time)
+// and 23 us at 128K, against 142 and about 60 us for the statistics, the vote
 // and the eight top-k launches it replaces.
 __global__ void __launch_bounds__(kVtThreads, 1) k_vote_topk(const VoteArgs a)
 {

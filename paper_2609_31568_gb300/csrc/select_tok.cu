@@ -25,8 +25,10 @@
 //                   owns its (unit, token) cells, so no atomics are needed.
 //
 // Each CTA owns a tile of 128 / g units and a range of 128 g tokens (<= 1024).
-// Calls of at most 16 units (every call of the Algorithm 2 loop) go to score.cu:
-// one read of K, planes of logits in the workspace. Where the planes do not
+// Calls over at most 16 sub-chunks (every call of the Algorithm 2 loop with outer
+// chunks of that length) go to score.cu: one read of K, planes of logits in the
+// workspace. The route and the order of the partial sums depend on the call, and
+// so do the last bits of the scores. Where the planes do not
 // fit there (small k with long sub-chunks) they use k_tok_score_s: 16 (unit,
 // head) columns per tile, tokens as the MMA rows and the three parts side by
 // side in one N = 48 operand.
@@ -834,7 +836,7 @@ cudaError_t launch_select_tokens(const Derived& d, int mode, int64_t tok_begin, 
     // fills later; where they do not fit (small k), K is read twice instead. Up
     // to 16 units the planes (8 H_q bytes per token and unit, written and read)
     // cost less than the second read of K per four units that they replace: one
-    // unit at 1M tokens 765 -> 397 us.
+    // unit at 1M tokens 765 -> 396 us.
     const int64_t z_stride = (d.N + 3) / 4 * 4;
     const size_t plane = static_cast<size_t>(d.Hq) * z_stride * sizeof(float);
     const size_t scratch_bytes = align_up(static_cast<size_t>(max_units) * kVoteScratchInts * sizeof(int32_t), kAlign);
